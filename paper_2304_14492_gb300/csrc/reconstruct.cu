@@ -364,48 +364,105 @@ __device__ __forceinline__ float pixel_rho(float x, float y, float cx, float cy,
     return sqrtf((*dx) * (*dx) + (*dy) * (*dy)) / r;
 }
 
+// Canvases of one launch in groups of one geometry: the images of a group share
+// every pixel's place on the polar grid.
+struct CartGroup {
+    int first, count;
+};
 struct CartParams {
     int n_rho, n_theta, b_off;
+    int gauss;              // Gauss-Legendre nodes (else the midpoint rule)
     const float* rho32;
     const float* polar;     // [batch][n_rho][n_theta]
+    CartGroup grp[KD_MAX_IMG];
     CanvasDesc cv[KD_MAX_IMG];
 };
 
+// The last node <= rho, or -1: a guess from the nodes' closed form (exact to
+// about one node; Gauss-Legendre nodes lie near (1 - cos(pi (i + 3/4) / (n + 1/2))) / 2),
+// moved until the table itself confirms it.
+__device__ __forceinline__ int last_node(const float* __restrict__ rho32, int n_rho, int gauss, float rho) {
+    const float x = gauss ? ((float)n_rho + 0.5f) * (2.f / 3.14159265f) * asinf(sqrtf(fminf(rho, 1.f))) - 0.75f
+                          : rho * (float)n_rho - 0.5f;
+    int g = min(max((int)floorf(x), 0), n_rho - 1);
+    while (g + 1 < n_rho && __ldg(&rho32[g + 1]) <= rho) ++g;
+    while (g >= 0 && __ldg(&rho32[g]) > rho) --g;
+    return g;
+}
+
+// Polar reconstruction -> pixels.  A warp takes a 32 x 4 block of pixels as
+// four 8 x 4 tiles (a pixel of each tile per thread): the bilinear corners of
+// a compact tile fall on few 128-byte lines wherever it lies on the disk (a
+// 32 x 1 run along a radius touches a line per pixel), and stores still fill
+// whole 32-byte sectors.  The place of a pixel on the grid (square root,
+// division, atan2, node lookup: about 100 instructions) is computed once and
+// used for every image of the group; with it per image, one pixel per thread
+// and a ten-step search over the nodes, three 3840 x 2160 bands took 133 us,
+// now 69 us (both cold, serialised).  Bound by the L1 wavefronts of the corner
+// loads (62 % busy) and instruction issue (56 %).
+constexpr int PTC_TILES = 4, PTC_GROUP = 4;
 __global__ void __launch_bounds__(256) k_polar_to_cart(const __grid_constant__ CartParams p) {
-    const CanvasDesc c = p.cv[blockIdx.z];
-    const int x = blockIdx.x * 32 + threadIdx.x;
-    const int y = blockIdx.y * 8 + threadIdx.y;
-    if (x >= c.w || y >= c.h) return;
-    float dx, dy;
-    const float rho = pixel_rho((float)x, (float)y, c.cx, c.cy, c.r, &dx, &dy);
-    float val = 0.f;
-    if (rho <= 1.f) {
-        float th = atan2f(dy, dx);
-        if (th < 0.f) th += kTwoPi;
-        const int n_rho = p.n_rho, N = p.n_theta;
-        int lo = 0, hi = n_rho;                 // first node > rho
-        while (lo < hi) {
-            const int mid = (lo + hi) >> 1;
-            if (__ldg(&p.rho32[mid]) > rho) hi = mid; else lo = mid + 1;
+    const CartGroup g = p.grp[blockIdx.z];
+    const CanvasDesc c = p.cv[g.first];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int y = blockIdx.y * 32 + warp * 4 + (lane >> 3);
+    const int xb = blockIdx.x * 32 + (lane & 7);
+    if (y >= c.h) return;
+    const int n_rho = p.n_rho, N = p.n_theta;
+    // per pixel: the corners' offsets and the two fractions; o0 < 0: outside the disk
+    int o0[PTC_TILES], o1[PTC_TILES], dk[PTC_TILES];
+    float s[PTC_TILES], t[PTC_TILES];
+    bool any = false;
+#pragma unroll
+    for (int j = 0; j < PTC_TILES; ++j) {
+        o0[j] = -1;
+        float dx, dy;
+        const float rho = pixel_rho((float)(xb + 8 * j), (float)y, c.cx, c.cy, c.r, &dx, &dy);
+        if (rho <= 1.f && xb + 8 * j < c.w) {
+            float th = atan2f(dy, dx);
+            if (th < 0.f) th += kTwoPi;
+            const int lo = last_node(p.rho32, n_rho, p.gauss, rho);
+            const int i1 = min(lo + 1, n_rho - 1), i0 = max(lo, 0);
+            const float r0 = __ldg(&p.rho32[i0]), r1 = __ldg(&p.rho32[i1]);
+            const float span = r1 - r0;
+            const float tt = span > 0.f ? (rho - r0) / span : 0.f;
+            t[j] = fminf(fmaxf(tt, 0.f), 1.f);
+            const float v = th * (float)N / kTwoPi;
+            const float kf = floorf(v);
+            s[j] = v - kf;
+            const int k0 = ((int)kf) & (N - 1);
+            dk[j] = ((k0 + 1) & (N - 1)) - k0;
+            o0[j] = i0 * N + k0;
+            o1[j] = i1 * N + k0;
+            any = true;
         }
-        const int i1 = min(lo, n_rho - 1);
-        const int i0 = max(min(lo - 1, n_rho - 1), 0);
-        const float r0 = __ldg(&p.rho32[i0]), r1 = __ldg(&p.rho32[i1]);
-        const float span = r1 - r0;
-        float t = span > 0.f ? (rho - r0) / span : 0.f;
-        t = fminf(fmaxf(t, 0.f), 1.f);
-        const float v = th * (float)N / kTwoPi;
-        const float kf = floorf(v);
-        const float s = v - kf;
-        const int k0 = ((int)kf) & (N - 1);
-        const int k1 = (k0 + 1) & (N - 1);
-        const float* pb = p.polar + (size_t)(p.b_off + blockIdx.z) * n_rho * N;
-        const float a0 = __ldg(&pb[(size_t)i0 * N + k0]), a1 = __ldg(&pb[(size_t)i0 * N + k1]);
-        const float b0 = __ldg(&pb[(size_t)i1 * N + k0]), b1 = __ldg(&pb[(size_t)i1 * N + k1]);
-        const float ra = fmaf(s, a1 - a0, a0), rb = fmaf(s, b1 - b0, b0);
-        val = fmaf(t, rb - ra, ra);
     }
-    c.data[(size_t)y * c.pitch + x] = val;
+    const size_t img = (size_t)n_rho * N;
+    const float* pb = p.polar + (size_t)(p.b_off + g.first) * img;
+    for (int q = 0; q < g.count; ++q, pb += img) {
+        float a0[PTC_TILES], a1[PTC_TILES], b0[PTC_TILES], b1[PTC_TILES];
+        if (any) {
+#pragma unroll
+            for (int j = 0; j < PTC_TILES; ++j)
+                if (o0[j] >= 0) {
+                    a0[j] = __ldg(pb + o0[j]);
+                    a1[j] = __ldg(pb + o0[j] + dk[j]);
+                    b0[j] = __ldg(pb + o1[j]);
+                    b1[j] = __ldg(pb + o1[j] + dk[j]);
+                }
+        }
+        float* row = p.cv[g.first + q].data + (size_t)y * p.cv[g.first + q].pitch;
+#pragma unroll
+        for (int j = 0; j < PTC_TILES; ++j) {
+            const int x = xb + 8 * j;
+            float val = 0.f;
+            if (o0[j] >= 0) {
+                const float ra = fmaf(s[j], a1[j] - a0[j], a0[j]), rb = fmaf(s[j], b1[j] - b0[j], b0[j]);
+                val = fmaf(t[j], rb - ra, ra);
+            }
+            if (x < c.w) row[x] = val;
+        }
+    }
 }
 
 static CanvasDesc resolve_canvas(const zm_canvas_t& cv) {
@@ -414,41 +471,94 @@ static CanvasDesc resolve_canvas(const zm_canvas_t& cv) {
     return CanvasDesc{cv.data, g.pitch, g.h, g.w, g.cx, g.cy, g.r};
 }
 
+static bool same_disk(const CanvasDesc& a, const CanvasDesc& b) {
+    return a.h == b.h && a.w == b.w && a.cx == b.cx && a.cy == b.cy && a.r == b.r;
+}
+
 int launch_polar_to_cart(zm_plan_t p, const float* polar, int batch, const zm_canvas_t* cv, cudaStream_t st) {
     static thread_local CartParams cp;
     cp.n_rho = p->n_rho;
     cp.n_theta = p->n_theta;
+    cp.gauss = (p->flags & ZM_GRID_GAUSS) ? 1 : 0;
     cp.rho32 = p->rho32;
     cp.polar = polar;
     for (int b0 = 0; b0 < batch; b0 += KD_MAX_IMG) {
         const int nb = std::min(KD_MAX_IMG, batch - b0);
         cp.b_off = b0;
-        int hmax = 1, wmax = 1;
+        int hmax = 1, wmax = 1, groups = 0;
         for (int j = 0; j < nb; ++j) {
             cp.cv[j] = resolve_canvas(cv[b0 + j]);
             hmax = std::max(hmax, cp.cv[j].h);
             wmax = std::max(wmax, cp.cv[j].w);
+            // up to four images a group: enough to spread the geometry's cost,
+            // and batches of small frames still fill the device
+            if (groups && cp.grp[groups - 1].count < PTC_GROUP && same_disk(cp.cv[cp.grp[groups - 1].first], cp.cv[j]))
+                ++cp.grp[groups - 1].count;
+            else
+                cp.grp[groups++] = CartGroup{j, 1};
         }
-        dim3 grid((wmax + 31) / 32, (hmax + 7) / 8, nb);
-        k_polar_to_cart<<<grid, dim3(32, 8), 0, st>>>(cp);
+        k_polar_to_cart<<<dim3((wmax + 8 * PTC_TILES - 1) / (8 * PTC_TILES), (hmax + 31) / 32, groups), 256, 0, st>>>(cp);
         ZM_LAUNCH_CHECK("k_polar_to_cart");
     }
     return ZM_OK;
 }
 
 // ============================================================== reductions
-constexpr int RED_BLOCKS = 64;
 constexpr int RED_THREADS = 256;
+constexpr int RED_WARPS = RED_THREADS / 32;
+constexpr int RED_PER_SM = 6;            // resident blocks per SM the registers allow
+constexpr int RED_SEG = 2048;            // polar nodes a warp takes at a time
+
+enum { RED_DISK_ERRORS = 0, RED_POLAR_ERRORS = 1, RED_DISK_MINMAX = 2 };
 
 struct RedParams {
-    int mode;                 // 0: errors over disk pixels, 1: errors over polar nodes, 2: min/max over disk
-    int n_nodes, b_off;
-    const float* fhat;        // mode 1
-    const float* frec;        // mode 1
-    double* part;             // [batch][RED_BLOCKS][4]
+    int n_nodes, b_off, nb;
+    const float* fhat;        // polar errors
+    const float* frec;
+    double* part;             // [image of the launch][gridDim.x][4]
+    int* done;                // blocks finished, 0 between launches
+    double* out;              // error modes: [batch][4]
+    float* mm;                // min / max: [batch][2]
     CanvasDesc ref[KD_MAX_IMG];
     CanvasDesc tst[KD_MAX_IMG];
 };
+
+// The columns [*xa, *xb) of row y whose centres lie in the disk (empty: 0, 0).
+// Membership is pixel_rho() <= 1 as everywhere (a not-a-number counts as
+// inside, as a per-pixel "> 1" test has it).  |dx| grows away from the column
+// nearest the centre and every float operation of pixel_rho() is monotone, so
+// the columns are one run around it; its ends are guessed from the circle and
+// moved until the test itself confirms them.
+__device__ __forceinline__ void disk_span(const CanvasDesc& c, int y, int* xa, int* xb) {
+    auto inside = [&](int x) {
+        float dx, dy;
+        return !(pixel_rho((float)x, (float)y, c.cx, c.cy, c.r, &dx, &dy) > 1.f);
+    };
+    *xa = *xb = 0;
+    const int last = c.w - 1;
+    const int xm = min((int)fminf(fmaxf(rintf(c.cx), 0.f), (float)last), last);
+    if (!inside(xm)) return;
+    const float dy = c.cy - (float)y;
+    const float hw = sqrtf(fmaxf(c.r * c.r - dy * dy, 0.f));
+    int a = min((int)fminf(fmaxf(ceilf(c.cx - hw), 0.f), (float)xm), xm);
+    int b = max(min((int)fminf(fmaxf(floorf(c.cx + hw), (float)xm), (float)last), last), xm);
+    while (a > 0 && inside(a - 1)) --a;
+    while (a < xm && !inside(a)) ++a;
+    while (b < last && inside(b + 1)) ++b;
+    while (b > xm && !inside(b)) --b;
+    *xa = a;
+    *xb = b + 1;
+}
+
+// Columns of a row as 16-byte words: [*va, *vb) relative to `row` is the
+// aligned middle of [xa, xb); up to three columns are left on either side.
+__device__ __forceinline__ void vector_span(const float* row, int xa, int xb, int* va, int* vb) {
+    const int phase = (int)((reinterpret_cast<uintptr_t>(row) >> 2) & 3);
+    const int a = xa + ((4 - ((xa + phase) & 3)) & 3);
+    const int n = xb > a ? (xb - a) & ~3 : 0;
+    *va = n ? a : xa;
+    *vb = n ? a + n : xa;
+}
 
 __device__ __forceinline__ float warp_sum(float v) {
     for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -463,108 +573,178 @@ __device__ __forceinline__ float warp_min(float v) {
     return v;
 }
 
-// Per block: (sum (f - g)^2, sum f^2, max f, count) for the error modes and
-// (min, max, -, count) for the min/max mode; float partials per thread, one
-// double record per block.
-__global__ void __launch_bounds__(RED_THREADS) k_reduce(const __grid_constant__ RedParams p) {
+// Sums over the disk's pixels or the polar nodes: (sum (f - g)^2, sum f^2,
+// max f, count) for the error modes, (min, max) for the min / max mode.  A warp
+// takes whole rows (runs of RED_SEG nodes), of which it reads only the disk's
+// columns, four 16-byte loads in flight per lane, with no test per pixel: bound
+// by memory.  Float partials per thread, one double record per block; the last
+// block to finish adds an image's records in a fixed order and writes the
+// result, so there is no second launch.  Three 3840 x 2160 bands: min / max
+// 151 + 5 us -> 19 us, errors 166 + 5 us -> 28 us (both cold, serialised; 44
+// and 88 MB read).  Before, 64 blocks an image tested every pixel with a
+// square root and a division and had one load in flight.
+template <int MODE>
+__global__ void __launch_bounds__(RED_THREADS, RED_PER_SM) k_reduce(const __grid_constant__ RedParams p) {
+    constexpr int U = MODE == RED_DISK_MINMAX ? 4 : 2;     // 16-byte loads in flight per lane and image
     const int bl = blockIdx.y;
     const int b = p.b_off + bl;
+    const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
     float s0 = 0.f, s1 = 0.f, mx = -INFINITY, mn = INFINITY;
-    float cnt = 0.f;
-    if (p.mode == 1) {
-        const float* f = p.fhat + (size_t)b * p.n_nodes;
-        const float* g = p.frec + (size_t)b * p.n_nodes;
-        for (int e = blockIdx.x * RED_THREADS + threadIdx.x; e < p.n_nodes; e += RED_BLOCKS * RED_THREADS) {
-            const float fv = __ldg(&f[e]);
-            const float d = fv - __ldg(&g[e]);
+    long long cnt = 0;
+    auto add = [&](float f, float g) {
+        if (MODE != RED_DISK_MINMAX) {
+            const float d = f - g;
             s0 = fmaf(d, d, s0);
-            s1 = fmaf(fv, fv, s1);
-            mx = fmaxf(mx, fv);
-            cnt += 1.f;
+            s1 = fmaf(f, f, s1);
+        } else {
+            mn = fminf(mn, f);
         }
-    } else {
-        const CanvasDesc c = p.ref[bl];
-        const CanvasDesc t = p.tst[bl];
-        for (int y = blockIdx.x; y < c.h; y += RED_BLOCKS) {
-            for (int x = threadIdx.x; x < c.w; x += RED_THREADS) {
-                float dx, dy;
-                if (pixel_rho((float)x, (float)y, c.cx, c.cy, c.r, &dx, &dy) > 1.f) continue;
-                const float fv = __ldg(&c.data[(size_t)y * c.pitch + x]);
-                if (p.mode == 0) {
-                    const float d = fv - __ldg(&t.data[(size_t)y * t.pitch + x]);
-                    s0 = fmaf(d, d, s0);
-                    s1 = fmaf(fv, fv, s1);
+        mx = fmaxf(mx, f);
+    };
+    const CanvasDesc& c = p.ref[bl];
+    const CanvasDesc& t = p.tst[bl];
+    const int rows = MODE == RED_POLAR_ERRORS ? (p.n_nodes + RED_SEG - 1) / RED_SEG : c.h;
+    const long long stride = gridDim.x * RED_WARPS;
+    for (long long y0 = blockIdx.x * RED_WARPS + w; y0 < rows; y0 += 32 * stride) {
+        // lane l: the span of the l-th of this warp's next 32 rows
+        int sa = 0, sb = 0;
+        if (MODE != RED_POLAR_ERRORS) {
+            if (y0 + l * stride < rows) disk_span(c, (int)(y0 + l * stride), &sa, &sb);
+        }
+        for (int q = 0; q < 32 && y0 + q * stride < rows; ++q) {
+            const int y = (int)(y0 + q * stride);
+            int xa, xb;
+            const float *f, *g;
+            if (MODE == RED_POLAR_ERRORS) {
+                xa = 0;
+                xb = min(RED_SEG, p.n_nodes - y * RED_SEG);
+                f = p.fhat + (size_t)b * p.n_nodes + (size_t)y * RED_SEG;
+                g = p.frec + (size_t)b * p.n_nodes + (size_t)y * RED_SEG;
+            } else {
+                xa = __shfl_sync(0xffffffffu, sa, q);
+                xb = __shfl_sync(0xffffffffu, sb, q);
+                f = c.data + (long long)y * c.pitch;
+                g = MODE == RED_DISK_ERRORS ? t.data + (long long)y * t.pitch : f;
+            }
+            if (xa >= xb) continue;
+            cnt += xb - xa;
+            int va, vb;
+            vector_span(f, xa, xb, &va, &vb);
+            // the columns outside the aligned middle: lane by lane
+            for (int x = xa + l; x < va; x += 32) add(__ldg(f + x), MODE != RED_DISK_MINMAX ? __ldg(g + x) : 0.f);
+            for (int x = vb + l; x < xb; x += 32) add(__ldg(f + x), MODE != RED_DISK_MINMAX ? __ldg(g + x) : 0.f);
+            const bool gvec = ((reinterpret_cast<uintptr_t>(g + va)) & 15) == 0;
+            const int nv = (vb - va) >> 2;
+            for (int v0 = l; v0 < nv; v0 += 32 * U) {
+                float4 fv[U], gv[U];
+#pragma unroll
+                for (int u = 0; u < U; ++u)
+                    if (v0 + 32 * u < nv) fv[u] = __ldg(reinterpret_cast<const float4*>(f + va) + v0 + 32 * u);
+#pragma unroll
+                for (int u = 0; u < U; ++u) gv[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (MODE != RED_DISK_MINMAX) {
+#pragma unroll
+                    for (int u = 0; u < U; ++u)
+                        if (v0 + 32 * u < nv) {
+                            const float* gp = g + va + 4 * (v0 + 32 * u);
+                            if (gvec) gv[u] = __ldg(reinterpret_cast<const float4*>(gp));
+                            else gv[u] = make_float4(__ldg(gp), __ldg(gp + 1), __ldg(gp + 2), __ldg(gp + 3));
+                        }
                 }
-                mx = fmaxf(mx, fv);
-                mn = fminf(mn, fv);
-                cnt += 1.f;
+#pragma unroll
+                for (int u = 0; u < U; ++u)
+                    if (v0 + 32 * u < nv) {
+                        add(fv[u].x, gv[u].x);
+                        add(fv[u].y, gv[u].y);
+                        add(fv[u].z, gv[u].z);
+                        add(fv[u].w, gv[u].w);
+                    }
             }
         }
     }
-    __shared__ float sh[4][RED_THREADS / 32];
-    const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+    __shared__ float sh[3][RED_WARPS];
+    __shared__ long long shc[RED_WARPS];
+    __shared__ int is_last;
     s0 = warp_sum(s0);
     s1 = warp_sum(s1);
     mx = warp_max(mx);
     mn = warp_min(mn);
-    cnt = warp_sum(cnt);
     if (l == 0) {
         sh[0][w] = s0;
-        sh[1][w] = p.mode == 2 ? mn : s1;
+        sh[1][w] = MODE == RED_DISK_MINMAX ? mn : s1;
         sh[2][w] = mx;
-        sh[3][w] = cnt;
+        shc[w] = cnt;
     }
     __syncthreads();
     if (threadIdx.x == 0) {
-        double a = 0, c1 = 0, c3 = 0;
-        float m2 = -INFINITY, m1 = INFINITY;
-        for (int j = 0; j < RED_THREADS / 32; ++j) {
+        double a = 0, c1 = MODE == RED_DISK_MINMAX ? (double)INFINITY : 0;
+        float m2 = -INFINITY;
+        long long n = 0;
+        for (int j = 0; j < RED_WARPS; ++j) {
             a += sh[0][j];
-            if (p.mode == 2) m1 = fminf(m1, sh[1][j]); else c1 += sh[1][j];
+            if (MODE == RED_DISK_MINMAX) c1 = fmin(c1, (double)sh[1][j]);
+            else c1 += sh[1][j];
             m2 = fmaxf(m2, sh[2][j]);
-            c3 += sh[3][j];
+            n += shc[j];
         }
-        double* o = p.part + ((size_t)b * RED_BLOCKS + blockIdx.x) * 4;
-        o[0] = a;
-        o[1] = p.mode == 2 ? (double)m1 : c1;
-        o[2] = (double)m2;
-        o[3] = c3;
+        double* o = p.part + ((size_t)bl * gridDim.x + blockIdx.x) * 4;
+        *reinterpret_cast<double2*>(o) = make_double2(a, c1);
+        *reinterpret_cast<double2*>(o + 2) = make_double2((double)m2, (double)n);
+        __threadfence();
+        is_last = atomicAdd(p.done, 1) == (int)(gridDim.x * gridDim.y) - 1;
     }
-}
-
-// mode 0/1: out[b] = (eps_1, eps, f_max, count) as doubles; mode 2: mm[b] = (min, max).
-// One warp per image: lanes take two block records each, then a shuffle tree
-// (few dependent double additions).
-__global__ void k_reduce_final(const double* __restrict__ part, int batch, int mode, double* __restrict__ out,
-                               float* __restrict__ mm) {
-    const int b = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    const int lane = threadIdx.x & 31;
-    if (b >= batch) return;
-    double sd = 0, sf = 0, cnt = 0, mx = -INFINITY, mn = INFINITY;
-    for (int j = lane; j < RED_BLOCKS; j += 32) {
-        const double* o = part + ((size_t)b * RED_BLOCKS + j) * 4;
-        sd += o[0];
-        if (mode == 2) mn = fmin(mn, o[1]); else sf += o[1];
-        mx = fmax(mx, o[2]);
-        cnt += o[3];
+    __syncthreads();
+    if (!is_last) return;
+    // out = (eps_1, eps, f_max, count), mm = (min, max): a warp per image,
+    // lanes over its records, then a shuffle tree
+    __threadfence();
+    for (int j = w; j < p.nb; j += RED_WARPS) {
+        double sd = 0, sf = 0, n = 0, dmx = -INFINITY, dmn = INFINITY;
+        const double2* rec = reinterpret_cast<const double2*>(p.part) + (size_t)j * gridDim.x * 2;
+        for (int e0 = l; e0 < (int)gridDim.x; e0 += 128) {      // four records in flight per lane
+            double2 ra[4], rb[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const bool on = e0 + 32 * u < (int)gridDim.x;
+                ra[u] = on ? __ldcg(rec + 2 * (e0 + 32 * u))
+                           : make_double2(0, MODE == RED_DISK_MINMAX ? (double)INFINITY : 0);
+                rb[u] = on ? __ldcg(rec + 2 * (e0 + 32 * u) + 1) : make_double2(-(double)INFINITY, 0);
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                if (MODE == RED_DISK_MINMAX) {
+                    dmn = fmin(dmn, ra[u].y);
+                } else {
+                    sd += ra[u].x;
+                    sf += ra[u].y;
+                    n += rb[u].y;
+                }
+                dmx = fmax(dmx, rb[u].x);
+            }
+        }
+        for (int o = 16; o; o >>= 1) {
+            if (MODE == RED_DISK_MINMAX) {
+                dmn = fmin(dmn, __shfl_xor_sync(0xffffffffu, dmn, o));
+            } else {
+                sd += __shfl_xor_sync(0xffffffffu, sd, o);
+                sf += __shfl_xor_sync(0xffffffffu, sf, o);
+                n += __shfl_xor_sync(0xffffffffu, n, o);
+            }
+            dmx = fmax(dmx, __shfl_xor_sync(0xffffffffu, dmx, o));
+        }
+        if (l) continue;
+        const size_t bj = (size_t)(p.b_off + j);
+        if (MODE == RED_DISK_MINMAX) {
+            p.mm[2 * bj] = (float)dmn;
+            p.mm[2 * bj + 1] = (float)dmx;
+        } else {
+            p.out[4 * bj + 0] = sd / sf;
+            p.out[4 * bj + 1] = sd / (dmx * dmx * n);
+            p.out[4 * bj + 2] = dmx;
+            p.out[4 * bj + 3] = n;
+        }
     }
-    for (int o = 16; o; o >>= 1) {
-        sd += __shfl_xor_sync(0xffffffffu, sd, o);
-        sf += __shfl_xor_sync(0xffffffffu, sf, o);
-        cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
-        mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-        mn = fmin(mn, __shfl_xor_sync(0xffffffffu, mn, o));
-    }
-    if (lane) return;
-    if (mode == 2) {
-        mm[2 * b] = (float)mn;
-        mm[2 * b + 1] = (float)mx;
-    } else {
-        out[4 * b + 0] = sd / sf;
-        out[4 * b + 1] = sd / (mx * mx * cnt);
-        out[4 * b + 2] = mx;
-        out[4 * b + 3] = cnt;
-    }
+    if (threadIdx.x == 0) *p.done = 0;
 }
 
 // out[b] = (eps_1, eps, f_max, count) from the nrec ring records (sd, sf,
@@ -621,44 +801,58 @@ k_reduce_records(const float4* __restrict__ part, int nrec, double count, double
     }
 }
 
-static int run_reduce(zm_plan_t p, int mode, const zm_image_t* ref, const zm_image_t* tst, const float* fhat,
+// Blocks per image of the row kernels: a row per warp where the device holds
+// that many at once (a second row for a few of the warps would double the
+// time), at least one block an image.
+static int row_blocks(zm_plan_t p, int rows, int nb) {
+    const int want = std::max(1, RED_PER_SM * num_sms(p->device) / nb);
+    return std::min(std::min(RED_MAX_BLOCKS, want), std::max(1, (rows + RED_WARPS - 1) / RED_WARPS));
+}
+
+template <int MODE>
+static int run_reduce(zm_plan_t p, const zm_image_t* ref, const zm_image_t* tst, const float* fhat,
                       const float* frec, int batch, double* out, float* mm, cudaStream_t st) {
-    int s = p->ws_red.grow(sizeof(double) * (size_t)batch * RED_BLOCKS * 4);
-    if (s != ZM_OK) return s;
     static thread_local RedParams rp;
-    rp.mode = mode;
     rp.n_nodes = p->n_rho * p->n_theta;
     rp.fhat = fhat;
     rp.frec = frec;
-    rp.part = (double*)p->ws_red.ptr;
+    rp.out = out;
+    rp.mm = mm;
+    rp.done = p->work + 2;
+    int s = p->ws_red.grow(sizeof(double) * 4 * RED_MAX_BLOCKS * (size_t)std::min(batch, KD_MAX_IMG));
+    if (s != ZM_OK) return s;
     for (int b0 = 0; b0 < batch; b0 += KD_MAX_IMG) {
         const int nb = std::min(KD_MAX_IMG, batch - b0);
         rp.b_off = b0;
-        if (mode != 1) {
+        rp.nb = nb;
+        int rows = MODE == RED_POLAR_ERRORS ? (rp.n_nodes + RED_SEG - 1) / RED_SEG : 1;
+        if (MODE != RED_POLAR_ERRORS) {
             for (int j = 0; j < nb; ++j) {
                 const GeoImage g = resolve(ref[b0 + j]);
                 rp.ref[j] = CanvasDesc{const_cast<float*>(g.data), g.pitch, g.h, g.w, g.cx, g.cy, g.r};
-                if (mode == 0) {
+                rows = std::max(rows, g.h);
+                if (MODE == RED_DISK_ERRORS) {
                     const GeoImage t = resolve(tst[b0 + j]);
                     rp.tst[j] = CanvasDesc{const_cast<float*>(t.data), t.pitch, t.h, t.w, t.cx, t.cy, t.r};
                 }
             }
         }
-        k_reduce<<<dim3(RED_BLOCKS, nb), RED_THREADS, 0, st>>>(rp);
+        const int blocks = row_blocks(p, rows, nb);
+        rp.part = (double*)p->ws_red.ptr;         // each launch finishes its own images
+        k_reduce<MODE><<<dim3(blocks, nb), RED_THREADS, 0, st>>>(rp);
         ZM_LAUNCH_CHECK("k_reduce");
     }
-    k_reduce_final<<<(batch + 3) / 4, 128, 0, st>>>((const double*)p->ws_red.ptr, batch, mode, out, mm);
-    ZM_LAUNCH_CHECK("k_reduce_final");
     return ZM_OK;
 }
 
 int launch_errors(zm_plan_t p, const zm_image_t* ref, const zm_image_t* test, const float* fhat,
                   const float* frec, int batch, double* out, cudaStream_t st) {
-    return run_reduce(p, fhat ? 1 : 0, ref, test, fhat, frec, batch, out, nullptr, st);
+    if (fhat) return run_reduce<RED_POLAR_ERRORS>(p, nullptr, nullptr, fhat, frec, batch, out, nullptr, st);
+    return run_reduce<RED_DISK_ERRORS>(p, ref, test, nullptr, nullptr, batch, out, nullptr, st);
 }
 
 int launch_disk_minmax(zm_plan_t p, const zm_image_t* imgs, int batch, float* out, cudaStream_t st) {
-    return run_reduce(p, 2, imgs, nullptr, nullptr, nullptr, batch, nullptr, out, st);
+    return run_reduce<RED_DISK_MINMAX>(p, imgs, nullptr, nullptr, nullptr, batch, nullptr, out, st);
 }
 
 struct NormParams {
@@ -668,19 +862,38 @@ struct NormParams {
     CanvasDesc cv[KD_MAX_IMG];
 };
 
-__global__ void __launch_bounds__(256) k_minmax_apply(const __grid_constant__ NormParams p) {
-    const CanvasDesc c = p.cv[blockIdx.z];
-    const int x = blockIdx.x * 32 + threadIdx.x;
-    const int y = blockIdx.y * 8 + threadIdx.y;
-    if (x >= c.w || y >= c.h) return;
-    float dx, dy;
-    if (pixel_rho((float)x, (float)y, c.cx, c.cy, c.r, &dx, &dy) > 1.f) return;
-    const int b = p.b_off + blockIdx.z;
+// Rows as in k_reduce: a warp per row, only the disk's columns, 16-byte loads
+// and stores, the scale once per warp (three 3840 x 2160 bands: 62 us with a
+// thread and a membership test per pixel, now 15 us, cold; 88 MB moved).
+__global__ void __launch_bounds__(RED_THREADS) k_minmax_apply(const __grid_constant__ NormParams p) {
+    const CanvasDesc& c = p.cv[blockIdx.y];
+    const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+    const int b = p.b_off + blockIdx.y;
     const float gmin = p.mm[2 * b], gmax = p.mm[2 * b + 1];
     const float lo = p.target[2 * b], hi = p.target[2 * b + 1];
     const float scale = gmax > gmin ? (hi - lo) / (gmax - gmin) : 0.f;
-    float* px = c.data + (size_t)y * c.pitch + x;
-    *px = fmaf(*px - gmin, scale, lo);
+    auto map = [&](float v) { return fmaf(v - gmin, scale, lo); };
+    for (long long yl = blockIdx.x * RED_WARPS + w; yl < c.h; yl += gridDim.x * RED_WARPS) {
+        const int y = (int)yl;
+        int xa, xb, va, vb;
+        disk_span(c, y, &xa, &xb);
+        if (xa >= xb) continue;
+        float* row = c.data + (long long)y * c.pitch;
+        vector_span(row, xa, xb, &va, &vb);
+        for (int x = xa + l; x < va; x += 32) row[x] = map(row[x]);
+        for (int x = vb + l; x < xb; x += 32) row[x] = map(row[x]);
+        float4* px = reinterpret_cast<float4*>(row + va);
+        const int nv = (vb - va) >> 2;
+        for (int v0 = l; v0 < nv; v0 += 128) {
+            float4 f[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (v0 + 32 * u < nv) f[u] = px[v0 + 32 * u];
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (v0 + 32 * u < nv) px[v0 + 32 * u] = make_float4(map(f[u].x), map(f[u].y), map(f[u].z), map(f[u].w));
+        }
+    }
 }
 
 int launch_minmax_normalize(zm_plan_t p, const zm_canvas_t* cv, int batch, const float* target, cudaStream_t st) {
@@ -690,7 +903,7 @@ int launch_minmax_normalize(zm_plan_t p, const zm_canvas_t* cv, int batch, const
     for (int b = 0; b < batch; ++b)
         ims[b] = zm_image_t{cv[b].data, cv[b].height, cv[b].width, cv[b].pitch, cv[b].cx, cv[b].cy, cv[b].radius};
     float* mm = (float*)p->ws_scale.ptr;
-    s = run_reduce(p, 2, ims.data(), nullptr, nullptr, nullptr, batch, nullptr, mm, st);
+    s = run_reduce<RED_DISK_MINMAX>(p, ims.data(), nullptr, nullptr, nullptr, batch, nullptr, mm, st);
     if (s != ZM_OK) return s;
     static thread_local NormParams np;
     np.mm = mm;
@@ -698,13 +911,12 @@ int launch_minmax_normalize(zm_plan_t p, const zm_canvas_t* cv, int batch, const
     for (int b0 = 0; b0 < batch; b0 += KD_MAX_IMG) {
         const int nb = std::min(KD_MAX_IMG, batch - b0);
         np.b_off = b0;
-        int hmax = 1, wmax = 1;
+        int hmax = 1;
         for (int j = 0; j < nb; ++j) {
             np.cv[j] = resolve_canvas(cv[b0 + j]);
             hmax = std::max(hmax, np.cv[j].h);
-            wmax = std::max(wmax, np.cv[j].w);
         }
-        k_minmax_apply<<<dim3((wmax + 31) / 32, (hmax + 7) / 8, nb), dim3(32, 8), 0, st>>>(np);
+        k_minmax_apply<<<dim3(row_blocks(p, hmax, nb), nb), RED_THREADS, 0, st>>>(np);
         ZM_LAUNCH_CHECK("k_minmax_apply");
     }
     return ZM_OK;

@@ -193,7 +193,8 @@ struct zm_plan_s {
     zm::Workspace ws_colmax;    // per-column max |F| (fp16 split scaling)
     zm::Workspace ws_Fblk;      // ring spectra as bf16 hi / lo operand blocks (blocked projection)
     int* status = nullptr;      // device status word: ZM_ETIMEOUT after a timed-out wait
-    int* work = nullptr;        // device {next item, CTAs done} of the inverse ring FFT, 0 between launches
+    int* work = nullptr;        // device {next item, CTAs done} of the inverse ring FFT and {blocks done} of the
+                                // reductions, 0 between launches
     // launch choices
     int kb_rings = 8;           // rings per CTA in the resample + FFT kernel
     // set by the batch autotuner (0 = built-in heuristic)
@@ -306,6 +307,8 @@ inline GeoImage resolve(const zm_image_t& im) {
 }
 
 int check_images(const zm_image_t* imgs, int batch);
+
+constexpr int RED_MAX_BLOCKS = 512;   // blocks (records) per image of the pixel and node reductions
 
 // Cartesian-tile resampling (resample_tiles.cu)
 bool tma_eligible(const zm_image_t& im);
