@@ -250,22 +250,13 @@ int zm_project(zm_plan_t plan, const float* spectra, int batch, float* out,
  * at call time: their device memory is already handed out by another
  * allocator (e.g. a framework's caching pool that reserved the GPU up front),
  * or they run in a loop where cudaMalloc's device-wide synchronisation and
- * unbounded latency are not acceptable.  It allocates nothing: the split-K
- * partial sums live in a fixed 8 MiB array in device memory that belongs to
- * the library (held by every GPU that loads it, until the process exits).
- * The paper has no counterpart; this is an interface matter only.
+ * unbounded latency are not acceptable.  It allocates nothing and keeps no
+ * device memory of its own: the sums stay on chip.  The paper has no
+ * counterpart; this is an interface matter only.
  *  - Computes in FP32 whatever the plan's precision flag; the plan itself is
  *    made beforehand with zm_plan (which does allocate).
  *  - Requires P(n_max) * 2 * batch <= 2^21 floats; larger requests return
  *    ZM_EINVAL without touching the device.
- *  - The first call on a device looks up the array's device address (set-up,
- *    with that device current); make that first call before any stream
- *    capture.  The address is kept for the process's lifetime: resetting the
- *    device (cudaDeviceReset) between calls is not supported.
- *  - All calls on a device share the array and it keeps the last call's
- *    contents; each call overwrites the part it reads, so nothing needs
- *    clearing, but calls that overlap on the GPU (other streams, other
- *    threads) race: serialise them.
  * Arguments, layouts and flags as zm_project. */
 int zm_project_noalloc(zm_plan_t plan, const float* spectra, int batch, float* out,
                        unsigned flags, void* stream);

@@ -254,6 +254,7 @@ static int tune_group(zm_batch_t b, BatchGroup& g, const zm_request_t* reqs,
     for (int gather = 0; gather <= (tma ? 1 : 0); ++gather)
         for (int rings : {2, 4, 8})
             for (int split : {4, 8}) {
+                if (split > 4 && g.plan->prec == PREC_FP32) continue;      // no radial split there
                 g.plan->tune_gather = gather;
                 g.plan->tune_rings = rings;
                 g.plan->tune_split = split;

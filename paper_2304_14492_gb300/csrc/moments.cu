@@ -427,130 +427,6 @@ static int launch_kb_mode(int logn, const KbParams& kp, int R, int nb, cudaStrea
     }
 }
 
-// ============================================================== K-c (FP32)
-// For each m: the (K_m x N_rho) x (N_rho x 2B) product
-//   D[n][col] = sum_i A[row(m,n)][i] F[m][col][i],   col = 2b + re/im,
-// split over i into S partial sums (part[s][row][col]); k_project_reduce adds
-// them in a fixed order and applies the Neumann factor.
-constexpr int KC_ROWS = 64, KC_COLS = 32, KC_K = 32;
-
-__global__ void __launch_bounds__(256)
-k_project_fp32(const float* __restrict__ A32, const float* __restrict__ F, const int* __restrict__ mrow,
-               int n_max, int n_rho, int ncol, int chunk, int P, float* __restrict__ part) {
-    __shared__ float As[KC_K][KC_ROWS + 1];
-    __shared__ float Fs[KC_K][KC_COLS + 1];
-    const int m = blockIdx.x;
-    const int col0 = blockIdx.y * KC_COLS;
-    const int s = blockIdx.z;
-    const int Km = (n_max - m) / 2 + 1;
-    const int rowbase = mrow[m];
-    const int ib = s * chunk, ie = min(n_rho, ib + chunk);
-    const int tid = threadIdx.x, ty = tid >> 3, tx = tid & 7;
-    const float* Fm = F + ((size_t)m * ncol + col0) * n_rho;
-    for (int rt = 0; rt < Km; rt += KC_ROWS) {
-        float acc[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
-        for (int kk = ib; kk < ie; kk += KC_K) {
-            for (int e = tid; e < KC_ROWS * KC_K; e += 256) {
-                const int row = e >> 5, k = e & 31;
-                const int gr = rt + row, gk = kk + k;
-                As[k][row] = (gr < Km && gk < ie) ? __ldg(&A32[(size_t)(rowbase + gr) * n_rho + gk]) : 0.f;
-            }
-            for (int e = tid; e < KC_COLS * KC_K; e += 256) {
-                const int col = e >> 5, k = e & 31;
-                const int gk = kk + k;
-                Fs[k][col] = (col0 + col < ncol && gk < ie) ? __ldg(&Fm[(size_t)col * n_rho + gk]) : 0.f;
-            }
-            __syncthreads();
-#pragma unroll 8
-            for (int k = 0; k < KC_K; ++k) {
-                const float a0 = As[k][2 * ty], a1 = As[k][2 * ty + 1];
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const float f = Fs[k][4 * tx + j];
-                    acc[0][j] = fmaf(a0, f, acc[0][j]);
-                    acc[1][j] = fmaf(a1, f, acc[1][j]);
-                }
-            }
-            __syncthreads();
-        }
-#pragma unroll
-        for (int a = 0; a < 2; ++a) {
-            const int gr = rt + 2 * ty + a;
-            if (gr >= Km) continue;
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const int col = col0 + 4 * tx + j;
-                if (col < ncol) part[((size_t)s * P + rowbase + gr) * ncol + col] = acc[a][j];
-            }
-        }
-    }
-}
-
-__global__ void k_project_reduce(const float* __restrict__ part, int S, int P, int ncol,
-                                 const int2* __restrict__ pair_nm, const int* __restrict__ mrow,
-                                 int batch, int neumann, float* __restrict__ out) {
-    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= batch * P) return;
-    const int b = idx / P, q = idx - b * P;
-    const int2 nm = pair_nm[q];
-    const int row = mrow[nm.y] + (nm.x - nm.y) / 2;
-    float re = 0.f, im = 0.f;
-    for (int s = 0; s < S; ++s) {
-        const float* ps = part + ((size_t)s * P + row) * ncol + 2 * b;
-        re += ps[0];
-        im += ps[1];
-    }
-    const float f = (neumann && nm.y == 0) ? 0.5f : 1.f;
-    out[(size_t)idx * 2] = re * f;
-    out[(size_t)idx * 2 + 1] = im * f;
-}
-
-// Radial split of the FP32 projection: S slices of `chunk` nodes (a multiple
-// of KC_K) aiming at the tuned number of CTAs per SM, at most max_slices of
-// them (re-deriving S from the chunk never raises it).
-static void fp32_split(zm_plan_t p, int batch, long long max_slices, int* S_out, int* chunk_out) {
-    const int ctiles = (2 * batch + KC_COLS - 1) / KC_COLS;
-    const int base = (p->n_max + 1) * ctiles;
-    const int target = (p->tune_split > 0 ? p->tune_split : 4) * num_sms(p->device);
-    const int kchunks = (p->n_rho + KC_K - 1) / KC_K;
-    long long S = std::max(1, std::min(kchunks, (target + base - 1) / base));
-    S = std::max(1ll, std::min(S, max_slices));
-    const int chunk = (int)((kchunks + S - 1) / S) * KC_K;
-    *S_out = (p->n_rho + chunk - 1) / chunk;
-    *chunk_out = chunk;
-}
-
-static int launch_projection_fp32(zm_plan_t p, const float* F, int batch, float* out, unsigned flags,
-                                  cudaStream_t st) {
-    int S, chunk;
-    fp32_split(p, batch, 1ll << 40, &S, &chunk);
-    const int st_ = p->ws_part.grow(sizeof(float) * (size_t)S * p->P * 2 * batch);
-    if (st_ != ZM_OK) return st_;
-    return launch_projection_fp32_parts(p, F, batch, out, flags, (float*)p->ws_part.ptr,
-                                        p->ws_part.bytes / sizeof(float), st);
-}
-
-int launch_projection_fp32_parts(zm_plan_t p, const float* F, int batch, float* out, unsigned flags, float* part,
-                                 size_t part_floats, cudaStream_t st) {
-    const int ncol = 2 * batch;
-    const size_t one_slice = (size_t)p->P * ncol;
-    if (one_slice > part_floats)
-        return set_error(ZM_EINVAL, "projection partial sums: %zu floats per slice, %zu available", one_slice,
-                         part_floats);
-    int S, chunk;
-    fp32_split(p, batch, (long long)(part_floats / one_slice), &S, &chunk);
-    const int ctiles = (ncol + KC_COLS - 1) / KC_COLS;
-    dim3 grid(p->n_max + 1, ctiles, S);
-    k_project_fp32<<<grid, 256, 0, st>>>(p->A32, F, p->mrow, p->n_max, p->n_rho, ncol,
-                                          chunk, p->P, part);
-    ZM_LAUNCH_CHECK("k_project_fp32");
-    const int tot = batch * p->P;
-    k_project_reduce<<<(tot + 255) / 256, 256, 0, st>>>(part, S, p->P, ncol, p->pair_nm, p->mrow, batch,
-                                                         (flags & ZM_NEUMANN) ? 1 : 0, out);
-    ZM_LAUNCH_CHECK("k_project_reduce");
-    return ZM_OK;
-}
-
 // ============================================================== driver
 static int pick_rings(zm_plan_t p, int batch) {
     if (p->tune_rings == 2 || p->tune_rings == 4 || p->tune_rings == 8) return p->tune_rings;
@@ -816,9 +692,9 @@ extern "C" int zm_plan_reserve(zm_plan_t plan, int batch) {
     int s = plan->ws_F.grow(sizeof(float) * (size_t)(plan->n_max + 1) * nb * 2 * plan->n_rho);
     // polar samples of the tile resampler
     if (s == ZM_OK) s = plan->ws_fhat.grow(sizeof(float) * nb * plan->n_rho * plan->n_theta);
-    // projection partials: the radial split never exceeds one slice per 32 nodes
-    const size_t S = (size_t)(plan->n_rho + KC_K - 1) / KC_K;
-    if (s == ZM_OK) s = plan->ws_part.grow(sizeof(float) * S * plan->P * 2 * nb);
+    // partial sums of the split-K tensor-core projection: never more than one slice per 32 nodes
+    const size_t S = (size_t)(plan->n_rho + 31) / 32;
+    if (s == ZM_OK && plan->prec != PREC_FP32) s = plan->ws_part.grow(sizeof(float) * S * plan->P * 2 * nb);
     if (s == ZM_OK) s = plan->ws_colmax.grow(sizeof(unsigned) * 2 * nb);
     if (s == ZM_OK) s = plan->ws_G.grow(sizeof(float) * g_floats(batch, plan->n_rho, plan->n_max));
     // reductions: a record per block of an image (pixel errors) or per ring (fused errors)
