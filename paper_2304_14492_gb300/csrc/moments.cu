@@ -695,7 +695,6 @@ extern "C" int zm_plan_reserve(zm_plan_t plan, int batch) {
     // partial sums of the split-K tensor-core projection: never more than one slice per 32 nodes
     const size_t S = (size_t)(plan->n_rho + 31) / 32;
     if (s == ZM_OK && plan->prec != PREC_FP32) s = plan->ws_part.grow(sizeof(float) * S * plan->P * 2 * nb);
-    if (s == ZM_OK) s = plan->ws_colmax.grow(sizeof(unsigned) * 2 * nb);
     if (s == ZM_OK) s = plan->ws_G.grow(sizeof(float) * g_floats(batch, plan->n_rho, plan->n_max));
     // reductions: a record per block of an image (pixel errors) or per ring (fused errors)
     const size_t rec = std::max<size_t>(RED_MAX_BLOCKS, (size_t)plan->n_rho);

@@ -44,30 +44,45 @@ struct TcParams {
     int ntmax;               // A tile rows reserved in shared memory (widest N of the launch)
     int fp16;                // 0: bf16 halves, 1: fp16 halves (scaled)
     float a_scale;           // A halves hold A * a_scale
-    const unsigned* colmax;  // fp16: per column max |F| (float bits); NULL = no scaling
 };
 
 // Power-of-two scale putting a column's largest |F| just below 2^14, so the
 // fp16 halves neither overflow nor lose the low part to subnormals.
-__device__ __forceinline__ float column_scale(const unsigned* colmax, int col) {
-    if (!colmax) return 1.f;
-    const float mx = __uint_as_float(colmax[col]);
+__device__ __forceinline__ float column_scale(float mx) {
     if (!(mx > 0.f) || !isfinite(mx)) return 1.f;
     int e;
     frexpf(mx, &e);
     return ldexpf(1.f, 14 - e);
 }
 
-// max |F[m][col][i]| over m and i, per column, as ordered float bits.
-__global__ void k_colmax(const float* __restrict__ F, int nm1, int ncol, int n_rho, unsigned* __restrict__ out) {
-    const int col = blockIdx.x;
-    float mx = 0.f;
-    for (int e = threadIdx.x + blockIdx.y * blockDim.x; e < nm1 * n_rho; e += blockDim.x * gridDim.y) {
-        const int m = e / n_rho, i = e - m * n_rho;
-        mx = fmaxf(mx, fabsf(__ldg(&F[((size_t)m * ncol + col) * n_rho + i])));
+// fp16: the scales of this CTA's columns over its own slice [ib, ie) of the
+// radius, eight threads a column.  A slice's partial sums leave the kernel
+// unscaled, so every slice can take its own scale; maxima over all m and nodes
+// needed a memset and a pass of their own (22 us of a 49 us call: five 1503 x
+// 1001 crops at n_max 80), here they are a second look at data the CTA loads
+// anyway.
+__device__ __forceinline__ void slice_scales(const float* Fm, int vrows, int col0, int n_rho, int ib, int ie, bool vec,
+                                             float* cscale) {
+    const int g = threadIdx.x & 7;
+    for (int r0 = 0; r0 < vrows; r0 += TC_THREADS / 8) {
+        const int row = r0 + (threadIdx.x >> 3);
+        float mx = 0.f;
+        if (row < vrows) {
+            const float* src = Fm + (size_t)(col0 + row) * n_rho;
+            if (vec && (ie & 3) == 0) {
+#pragma unroll 4
+                for (int k = ib + 4 * g; k < ie; k += 32) {
+                    const float4 v = __ldg(reinterpret_cast<const float4*>(src + k));
+                    mx = fmaxf(fmaxf(mx, fmaxf(fabsf(v.x), fabsf(v.y))), fmaxf(fabsf(v.z), fabsf(v.w)));
+                }
+            } else {
+#pragma unroll 4
+                for (int k = ib + g; k < ie; k += 8) mx = fmaxf(mx, fabsf(__ldg(src + k)));
+            }
+        }
+        for (int o = 4; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+        if (g == 0 && row < vrows) cscale[row] = column_scale(mx);
     }
-    for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    if ((threadIdx.x & 31) == 0) atomicMax(out + col, __float_as_uint(mx));
 }
 
 __global__ void __launch_bounds__(TC_THREADS) k_project_tc(const __grid_constant__ TcParams p) {
@@ -110,9 +125,16 @@ __global__ void __launch_bounds__(TC_THREADS) k_project_tc(const __grid_constant
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = *tslot;
 
+    __shared__ float cscale[TC_M];
+    griddep_wait();                    // F is written, the partial sums are free
+    griddep_launch();
     const float* Fm = p.F + (size_t)m * p.ncol * p.n_rho;
-    const bool fvec = (p.n_rho & 3) == 0;
+    const bool fvec = (p.n_rho & 3) == 0 && (reinterpret_cast<uintptr_t>(p.F) & 15) == 0;
     const bool avec = (p.n_rho & 7) == 0;
+    if (p.fp16) {
+        slice_scales(Fm, vrows, col0, p.n_rho, ib, ie, fvec, cscale);
+        __syncthreads();
+    }
     const unsigned long long t0 = global_ns();
     uint32_t phase = 0;
     bool ok = true;
@@ -144,7 +166,7 @@ __global__ void __launch_bounds__(TC_THREADS) k_project_tc(const __grid_constant
                         for (int e = 0; e < 8; ++e) x[e] = (kk + e < ie) ? __ldg(src + e) : 0.f;
                     }
                 }
-                const float fs = column_scale(p.colmax, col);
+                const float fs = p.fp16 ? cscale[row] : 1.f;
                 uint16_t h[8], l[8];
 #pragma unroll
                 for (int e = 0; e < 8; ++e) split2(x[e] * fs, p.fp16, &h[e], &l[e]);
@@ -222,7 +244,7 @@ __global__ void __launch_bounds__(TC_THREADS) k_project_tc(const __grid_constant
         if (!ok) break;
         // epilogue: lanes 32w..32w+31 of TMEM = D rows (image columns)
         const int col = col0 + warp * 32 + lane;
-        const float inv = (col < p.ncol) ? 1.0f / (p.a_scale * column_scale(p.colmax, col)) : 0.f;
+        const float inv = (col < p.ncol) ? 1.0f / (p.a_scale * (p.fp16 ? cscale[warp * 32 + lane] : 1.f)) : 0.f;
         for (int c0 = 0; c0 < NT; c0 += 16) {
             uint32_t r[16];
             const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0;
@@ -263,11 +285,14 @@ __global__ void k_project_reduce_tc(const float* __restrict__ part, int S, int P
                                     const int2* __restrict__ pair_nm, const int* __restrict__ mrow, int batch,
                                     int neumann, float* __restrict__ out) {
     const int idx = blockIdx.x * blockDim.x + threadIdx.x;
+    griddep_wait();                    // the partial sums are written, out is free
+    griddep_launch();
     if (idx >= batch * P) return;
     const int b = idx / P, q = idx - b * P;
     const int2 nm = pair_nm[q];
     const int row = mrow[nm.y] + (nm.x - nm.y) / 2;
     float re = 0.f, im = 0.f;
+#pragma unroll 8
     for (int s = 0; s < S; ++s) {
         const float* ps = part + ((size_t)s * P + row) * ncol + 2 * b;
         re += ps[0];
@@ -281,16 +306,6 @@ __global__ void k_project_reduce_tc(const float* __restrict__ part, int S, int P
 int launch_projection_tc(zm_plan_t p, const float* F, int batch, float* out, unsigned flags, cudaStream_t st) {
     if (!p->Ahi || !p->Alo) return set_error(ZM_EINVAL, "plan has no tensor-core operands");
     const int ncol = 2 * batch;
-    int s = ZM_OK;
-    const unsigned* colmax = nullptr;
-    if (p->prec == PREC_FP16X3) {
-        s = p->ws_colmax.grow(sizeof(unsigned) * (size_t)ncol);
-        if (s != ZM_OK) return s;
-        ZM_CUDA_TRY(cudaMemsetAsync(p->ws_colmax.ptr, 0, sizeof(unsigned) * (size_t)ncol, st));
-        k_colmax<<<dim3(ncol, 4), 256, 0, st>>>(F, p->n_max + 1, ncol, p->n_rho, (unsigned*)p->ws_colmax.ptr);
-        ZM_LAUNCH_CHECK("k_colmax");
-        colmax = (const unsigned*)p->ws_colmax.ptr;
-    }
     const int ctiles = (ncol + TC_M - 1) / TC_M;
     const int base = (p->n_max + 1) * ctiles;
     // enough CTAs to cover the load -> MMA latency: up to one 64-wide chunk of
@@ -300,7 +315,7 @@ int launch_projection_tc(zm_plan_t p, const float* F, int batch, float* out, uns
     int S = std::max(1, std::min(std::min(kchunks, 32), (target + base - 1) / base));
     const int chunk = ((kchunks + S - 1) / S) * TC_KC;
     S = (p->n_rho + chunk - 1) / chunk;
-    s = p->ws_part.grow(sizeof(float) * (size_t)S * p->P * ncol);
+    const int s = p->ws_part.grow(sizeof(float) * (size_t)S * p->P * ncol);
     if (s != ZM_OK) return s;
     TcParams tp;
     tp.F = F;
@@ -316,7 +331,6 @@ int launch_projection_tc(zm_plan_t p, const float* F, int batch, float* out, uns
     tp.chunk = chunk;
     tp.fp16 = p->prec == PREC_FP16X3 ? 1 : 0;
     tp.a_scale = p->a_scale;
-    tp.colmax = colmax;
     // Shared memory also caps the resident CTAs so that their TMEM columns
     // (<= 256 each) never exceed the SM's 512.
     const int Km0 = p->n_max / 2 + 1;
@@ -335,12 +349,11 @@ int launch_projection_tc(zm_plan_t p, const float* F, int batch, float* out, uns
         if (dev < 64) configured[dev] = smem;
     }
     dim3 grid(p->n_max + 1, ctiles, S);
-    k_project_tc<<<grid, TC_THREADS, smem, st>>>(tp);
-    ZM_LAUNCH_CHECK("k_project_tc");
+    ZM_LAUNCH_PDL("k_project_tc", k_project_tc, grid, dim3(TC_THREADS), smem, st, tp);
     const int tot = batch * p->P;
-    k_project_reduce_tc<<<(tot + 255) / 256, 256, 0, st>>>(tp.part, S, p->P, ncol, p->pair_nm, p->mrow, batch,
-                                                            (flags & ZM_NEUMANN) ? 1 : 0, out);
-    ZM_LAUNCH_CHECK("k_project_reduce_tc");
+    ZM_LAUNCH_PDL("k_project_reduce_tc", k_project_reduce_tc, dim3((tot + 255) / 256), dim3(256), 0, st,
+                  (const float*)tp.part, S, p->P, ncol, (const int2*)p->pair_nm, (const int*)p->mrow, batch,
+                  (flags & ZM_NEUMANN) ? 1 : 0, out);
     return ZM_OK;
 }
 

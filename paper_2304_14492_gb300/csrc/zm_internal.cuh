@@ -190,7 +190,6 @@ struct zm_plan_s {
     zm::Workspace ws_G;         // reconstruction radial spectra G[b][m][2][n_rho]
     zm::Workspace ws_red;       // reduction partials
     zm::Workspace ws_scale;     // per-image min / max (normalisation)
-    zm::Workspace ws_colmax;    // per-column max |F| (fp16 split scaling)
     zm::Workspace ws_Fblk;      // ring spectra as bf16 hi / lo operand blocks (blocked projection)
     int* status = nullptr;      // device status word: ZM_ETIMEOUT after a timed-out wait
     int* work = nullptr;        // device {next item, CTAs done} of the inverse ring FFT and {blocks done} of the
