@@ -33,6 +33,7 @@
 #include <algorithm>
 #include <cmath>
 
+#include "packed.cuh"
 #include "zm_internal.cuh"
 
 namespace zm {
@@ -71,37 +72,6 @@ __device__ __forceinline__ float pix(const CsImage& g, int col, int row) {
                ? __ldg(g.data + (long long)row * g.pitch + col)
                : 0.f;
 }
-
-// two FP32 values in one register pair
-typedef unsigned long long f32x2;
-__device__ __forceinline__ f32x2 pack2(float a, float b) {
-    f32x2 r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-    return r;
-}
-__device__ __forceinline__ float2 unpack2(f32x2 v) {
-    float2 r;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
-    return r;
-}
-__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
-    f32x2 r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-    return r;
-}
-__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
-    f32x2 r;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
-    f32x2 r;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-constexpr f32x2 CS_MINUS1 = 0xbf800000bf800000ull;      // (-1, -1)
-__device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b) { return fma2(b, CS_MINUS1, a); }
-__device__ __forceinline__ f32x2 neg2(f32x2 a) { return mul2(a, CS_MINUS1); }
 
 // (x - j y)^m by repeated squaring from the highest bit of m, of two points at once
 __device__ __forceinline__ void cpow_conj(f32x2 x, f32x2 y, int m, f32x2* re, f32x2* im) {

@@ -6,6 +6,7 @@
 #include <map>
 #include <mutex>
 
+#include "packed.cuh"
 #include "ring_fft.cuh"
 #include "zm_internal.cuh"
 
@@ -17,64 +18,118 @@ constexpr float kTwoPi = 6.28318530717958647692f;
 // ============================================================== radial part
 // G(b, i, m, re/im) = c_m sum_{n = m, m+2, ..} R_nm(rho_i) Z_nm (layout g_index), with
 // c_m = 2/eps_m (c_0 = 1, c_m = 2) for the literal Eq. 9 and c_m = 1 for the
-// half sum over the stored m >= 0.  One thread = one node i, one m and RB
-// images (their moments staged in shared memory), so each table value is
-// read once per RB images.
-constexpr int RB = 8;
+// half sum over the stored m >= 0.
+//
+// Bound by reading the table once per RB images.  One CTA = 128 nodes, one m
+// and RB images (the fewest of 1, 2, 4, 8 that hold the batch); its eight warps
+// take every eighth order, so the longest chain is K_m / 8 steps and the few
+// heavy m do not outlast the rest, and their sums meet in shared memory in a
+// fixed order.  Each warp streams its own orders' rows through a ring of three
+// stages (cp.async, twelve rows in flight, the first ones on their way before
+// the moments are read); a lane multiplies two pairs of nodes (fma.rn.f32x2)
+// with moments staged twice each, so nothing is shuffled into pairs.  4 images,
+// n_max 500, 512 nodes (129 MB of table), cold: 68 us for a thread per node
+// with all K_m orders and eight image slots; 52 us with eight row loads held in
+// registers (104 of them, two CTAs per SM); 41 us like this.
+constexpr int RR_NODES = 128, RR_WARPS = 8, RR_U = 4, RR_STAGES = 3;
+constexpr int RR_RING = RR_STAGES * RR_U * RR_NODES;      // floats of a warp's ring
 
-__global__ void __launch_bounds__(128)
+// V: floats per copy (4, or 1 where rows are not 16-byte aligned).
+template <int RB, int V>
+__global__ void __launch_bounds__(32 * RR_WARPS, RB <= 4 ? 3 : 2)
 k_recon_radial(const float* __restrict__ R32m, const float2* __restrict__ Z, const int* __restrict__ mrow,
                int n_max, int n_rho, int P, int batch, int neumann, float* __restrict__ G) {
-    extern __shared__ float2 zs[];                 // [RB][Km]
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    extern __shared__ __align__(16) float rr_sm[];        // the rings, then the moments [RB][Km] (twice each)
+    const int i0 = blockIdx.x * RR_NODES;
     const int m = blockIdx.y;
     const int b0 = blockIdx.z * RB;
     const int nb = min(RB, batch - b0);
     const int Km = (n_max - m) / 2 + 1;
-    const int row0 = mrow[m];
-    for (int t = threadIdx.x; t < RB * Km; t += blockDim.x) {
-        const int bb = t / Km, j = t - bb * Km;
-        zs[t] = (bb < nb) ? __ldg(&Z[(size_t)(b0 + bb) * P + moment_index(m + 2 * j, m)]) : make_float2(0.f, 0.f);
-    }
-    __syncthreads();
-    if (i >= n_rho) return;
-    float re[RB], im[RB];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    float* ring = rr_sm + warp * RR_RING;
+    float4* zs4 = reinterpret_cast<float4*>(rr_sm + max(RR_WARPS * RR_RING, RR_WARPS * RB * 2 * RR_NODES));
+    const uint32_t ring_a = static_cast<uint32_t>(__cvta_generic_to_shared(ring));
+    const float* Rm = R32m + (size_t)mrow[m] * n_rho + i0;
+    auto issue = [&](int c, int st) {
 #pragma unroll
-    for (int bb = 0; bb < RB; ++bb) re[bb] = im[bb] = 0.f;
-    // eight table loads in flight per step: the loop is bound by their latency otherwise
-    const float* Rcol = R32m + (size_t)row0 * n_rho + i;
-    int j = 0;
-    for (; j + 8 <= Km; j += 8) {
-        float r[8];
+        for (int u = 0; u < RR_U; ++u) {
+            const int j = warp + RR_WARPS * (RR_U * c + u);
+            if (j >= Km) break;
+            const float* src = Rm + (size_t)j * n_rho;
+            const uint32_t dst = ring_a + 4u * (st * RR_U + u) * RR_NODES;
+            if (V == 4) {
+                const int on = i0 + 4 * lane < n_rho;     // else zero-filled
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst + 16u * lane),
+                             "l"(on ? src + 4 * lane : Rm), "r"(on ? 16 : 0) : "memory");
+            } else {
 #pragma unroll
-        for (int u = 0; u < 8; ++u) r[u] = __ldg(Rcol + (size_t)(j + u) * n_rho);
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-#pragma unroll
-            for (int bb = 0; bb < RB; ++bb) {
-                const float2 z = zs[bb * Km + j + u];
-                re[bb] = fmaf(r[u], z.x, re[bb]);
-                im[bb] = fmaf(r[u], z.y, im[bb]);
+                for (int e = 0; e < 4; ++e) {
+                    const int on = i0 + lane + 32 * e < n_rho;
+                    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst + 4u * (lane + 32 * e)),
+                                 "l"(on ? src + lane + 32 * e : Rm), "r"(on ? 4 : 0) : "memory");
+                }
             }
         }
-    }
-    for (; j < Km; ++j) {
-        const float r = __ldg(Rcol + (size_t)j * n_rho);
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
 #pragma unroll
-        for (int bb = 0; bb < RB; ++bb) {
-            const float2 z = zs[bb * Km + j];
-            re[bb] = fmaf(r, z.x, re[bb]);
-            im[bb] = fmaf(r, z.y, im[bb]);
-        }
+    for (int c = 0; c < RR_STAGES; ++c) issue(c, c);      // the table is the plan's
+    griddep_wait();                    // the moments are written, G is free
+    griddep_launch();
+    for (int t = threadIdx.x; t < RB * Km; t += blockDim.x) {
+        const int bb = t / Km, j = t - bb * Km;
+        const float2 z = (bb < nb) ? __ldg(&Z[(size_t)(b0 + bb) * P + moment_index(m + 2 * j, m)]) : make_float2(0.f, 0.f);
+        zs4[t] = make_float4(z.x, z.x, z.y, z.y);
     }
-    const float c = (neumann && m > 0) ? 2.f : 1.f;
+    __syncthreads();
+    f32x2 re[RB][2], im[RB][2];
 #pragma unroll
-    for (int bb = 0; bb < RB; ++bb) {
-        if (bb < nb) {
-            const int nrb = (n_rho + 7) / 8;
-            G[g_index(b0 + bb, i, m, 0, nrb, n_max + 1)] = c * re[bb];
-            G[g_index(b0 + bb, i, m, 1, nrb, n_max + 1)] = c * im[bb];
+    for (int bb = 0; bb < RB; ++bb) re[bb][0] = re[bb][1] = im[bb][0] = im[bb][1] = 0;
+    const ulonglong2* zs = reinterpret_cast<const ulonglong2*>(zs4);
+    int st = 0;
+    for (int c = 0; warp + RR_WARPS * RR_U * c < Km; ++c) {
+        asm volatile("cp.async.wait_group %0;" ::"n"(RR_STAGES - 1) : "memory");
+        __syncwarp();
+#pragma unroll
+        for (int u = 0; u < RR_U; ++u) {
+            const int j = warp + RR_WARPS * (RR_U * c + u);
+            if (j >= Km) break;
+            const ulonglong2 r = *reinterpret_cast<const ulonglong2*>(ring + (st * RR_U + u) * RR_NODES + 4 * lane);
+#pragma unroll
+            for (int bb = 0; bb < RB; ++bb) {
+                const ulonglong2 z = zs[bb * Km + j];
+                re[bb][0] = fma2(r.x, z.x, re[bb][0]);
+                re[bb][1] = fma2(r.y, z.x, re[bb][1]);
+                im[bb][0] = fma2(r.x, z.y, im[bb][0]);
+                im[bb][1] = fma2(r.y, z.y, im[bb][1]);
+            }
         }
+        __syncwarp();
+        issue(c + RR_STAGES, st);
+        st = st + 1 < RR_STAGES ? st + 1 : 0;
+    }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncthreads();                   // every ring is read: their place takes the sums
+    // sums [warp][image][re/im][node]
+    constexpr int OUT = RB * 2 * RR_NODES;
+#pragma unroll
+    for (int bb = 0; bb < RB; ++bb)
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+            const float2 a = unpack2(c ? im[bb][0] : re[bb][0]), b = unpack2(c ? im[bb][1] : re[bb][1]);
+            *reinterpret_cast<float4*>(rr_sm + warp * OUT + (bb * 2 + c) * RR_NODES + 4 * lane) =
+                make_float4(a.x, a.y, b.x, b.y);
+        }
+    __syncthreads();
+    const float cm = (neumann && m > 0) ? 2.f : 1.f;
+    const int nrb = (n_rho + 7) / 8;
+    const int parts = min(RR_WARPS, Km);
+    for (int e = threadIdx.x; e < OUT; e += blockDim.x) {
+        const int i = i0 + (e & (RR_NODES - 1)), bc = e / RR_NODES;
+        if (i >= n_rho || (bc >> 1) >= nb) continue;
+        float v = 0.f;
+        for (int w = 0; w < parts; ++w) v += rr_sm[w * OUT + e];
+        G[g_index(b0 + (bc >> 1), i, m, bc & 1, nrb, n_max + 1)] = cm * v;
     }
 }
 
@@ -289,6 +344,30 @@ static int launch_ifft(zm_plan_t p, const float* G, int batch, float* out, const
     }
 }
 
+template <int RB, int V>
+static int launch_radial_t(zm_plan_t p, const float* moments, int batch, unsigned flags, float* G, cudaStream_t st) {
+    const size_t smem = sizeof(float) * RR_WARPS * std::max(RR_RING, RB * 2 * RR_NODES) +
+                        sizeof(float4) * RB * (size_t)(p->n_max / 2 + 1);
+    const int dev = p->device;
+    static size_t configured[64] = {0};
+    if (smem > 48 * 1024 && (dev >= 64 || smem > configured[dev])) {
+        ZM_CUDA_TRY(
+            cudaFuncSetAttribute(k_recon_radial<RB, V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        if (dev < 64) configured[dev] = smem;
+    }
+    const int nz = (batch + RB - 1) / RB;
+    for (int z0 = 0; z0 < nz; z0 += 65535) {
+        const int nzc = std::min(65535, nz - z0);
+        const int b0 = z0 * RB;
+        const int nbc = std::min(batch - b0, nzc * RB);
+        ZM_LAUNCH_PDL("k_recon_radial", (k_recon_radial<RB, V>),
+                      dim3((p->n_rho + RR_NODES - 1) / RR_NODES, p->n_max + 1, nzc), dim3(32 * RR_WARPS), smem, st,
+                      (const float*)p->R32m, (const float2*)moments + (size_t)b0 * p->P, (const int*)p->mrow, p->n_max,
+                      p->n_rho, p->P, nbc, (flags & ZM_NEUMANN) ? 1 : 0, G + g_floats(b0, p->n_rho, p->n_max));
+    }
+    return ZM_OK;
+}
+
 static int launch_radial(zm_plan_t p, const float* moments, int batch, unsigned flags, cudaStream_t st,
                          float** G_out) {
     const int s = p->ws_G.grow(sizeof(float) * g_floats(batch, p->n_rho, p->n_max));
@@ -298,24 +377,12 @@ static int launch_radial(zm_plan_t p, const float* moments, int batch, unsigned 
         *G_out = G;
         return launch_radial_tc(p, moments, batch, flags, G, st);
     }
-    const size_t smem = sizeof(float2) * RB * (size_t)(p->n_max / 2 + 1);
-    int dev = p->device;
-    static size_t configured[64] = {0};
-    if (smem > 48 * 1024 && (dev >= 64 || smem > configured[dev])) {
-        ZM_CUDA_TRY(cudaFuncSetAttribute(k_recon_radial, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        if (dev < 64) configured[dev] = smem;
-    }
-    const int nz = (batch + RB - 1) / RB;
-    for (int z0 = 0; z0 < nz; z0 += 65535) {
-        const int nzc = std::min(65535, nz - z0);
-        const int b0 = z0 * RB;
-        const int nbc = std::min(batch - b0, nzc * RB);
-        dim3 grid((p->n_rho + 127) / 128, p->n_max + 1, nzc);
-        k_recon_radial<<<grid, 128, smem, st>>>(p->R32m, (const float2*)moments + (size_t)b0 * p->P, p->mrow,
-                                                 p->n_max, p->n_rho, p->P, nbc, (flags & ZM_NEUMANN) ? 1 : 0,
-                                                 G + g_floats(b0, p->n_rho, p->n_max));
-        ZM_LAUNCH_CHECK("k_recon_radial");
-    }
+    const bool vec = (p->n_rho & 3) == 0;
+    const int st_ = batch == 1   ? (vec ? launch_radial_t<1, 4> : launch_radial_t<1, 1>)(p, moments, batch, flags, G, st)
+                    : batch == 2 ? (vec ? launch_radial_t<2, 4> : launch_radial_t<2, 1>)(p, moments, batch, flags, G, st)
+                    : batch <= 4 ? (vec ? launch_radial_t<4, 4> : launch_radial_t<4, 1>)(p, moments, batch, flags, G, st)
+                                 : (vec ? launch_radial_t<8, 4> : launch_radial_t<8, 1>)(p, moments, batch, flags, G, st);
+    if (st_ != ZM_OK) return st_;
     *G_out = G;
     return ZM_OK;
 }
