@@ -151,10 +151,27 @@ def _ptr(x):
     raise TypeError("cannot take a device pointer of %r" % type(x))
 
 
+_raw_stream = None
+
+
+def _current_stream():
+    """torch's current stream as a raw cudaStream_t.  The first call goes through
+    torch.cuda.current_stream(), which initialises CUDA; later ones ask for the
+    handle alone (0.3 us where building the Stream object took 3.0 of a call's
+    10 us on the host)."""
+    global _raw_stream
+    if _raw_stream is None:
+        import torch
+        s = torch.cuda.current_stream().cuda_stream
+        get, dev = getattr(torch._C, "_cuda_getCurrentRawStream", None), getattr(torch._C, "_cuda_getDevice", None)
+        _raw_stream = (lambda: get(dev())) if get and dev else (lambda: torch.cuda.current_stream().cuda_stream)
+        return s
+    return _raw_stream()
+
+
 def _stream(s):
     if s is None:
-        import torch
-        return torch.cuda.current_stream().cuda_stream
+        return _current_stream()
     if isinstance(s, int):
         return s
     return s.cuda_stream
