@@ -146,12 +146,15 @@ int zm_plan_nodes(zm_plan_t plan, double* rho, double* wr, void* stream);
  *  imgs  host array of `batch` device image descriptors (any sizes)
  *  out   device float[batch][P][2]
  *  flags ZM_NEUMANN divides each moment by eps_m (2 for m = 0, else 1; Eq. 14)
- * Path: images with a 16-byte aligned base and a pitch and width that are
- * multiples of 4 floats are resampled and ring-transformed in one kernel (the
- * polar samples stay on chip) when a plan has at most 2^17 polar samples per
- * image, where that kernel measured faster; larger grids resample by image
- * tiles into a workspace first.  Both paths give the same moments, bit for
- * bit.  The environment variable ZM_FUSED, read when a plan is created,
+ * Path: grids of at most 256 angles, and smaller calls on 512, are resampled
+ * and ring-transformed in one kernel that gathers the pixels of each sample.
+ * Otherwise, images with a 16-byte aligned base and a pitch and width that are
+ * multiples of 4 floats are resampled and ring-transformed in one kernel that
+ * stages their rows (the polar samples stay on chip either way) when a plan has
+ * at most 2^17 polar samples per image, where that kernel measured faster;
+ * larger grids resample by image tiles into a workspace first.  All paths give
+ * the same moments, bit for bit.  The environment variable ZM_FUSED, read when
+ * a plan is created,
  * overrides the choice: "1" fuses wherever the geometry fits the kernel's
  * stage buffers, "0" never fuses.  ZM_RING_DFT=1, read likewise, sends bf16x3
  * plans with n_max <= 127 to a third kernel that resamples and computes the

@@ -242,7 +242,7 @@ static int tune_group(zm_batch_t b, BatchGroup& g, const zm_request_t* reqs,
     const std::string key = tune_key(g.plan, (int)g.members.size(), geo);
     auto it = cache.find(key);
     if (it != cache.end()) {
-        g.plan->tune_gather = it->second.gather;
+        g.plan->tune_gather = it->second.gather ? 1 : 2;
         g.plan->tune_rings = it->second.rings;
         g.plan->tune_split = it->second.split;
         return ZM_OK;
@@ -255,7 +255,7 @@ static int tune_group(zm_batch_t b, BatchGroup& g, const zm_request_t* reqs,
         for (int rings : {2, 4, 8})
             for (int split : {4, 8}) {
                 if (split > 4 && g.plan->prec == PREC_FP32) continue;      // no radial split there
-                g.plan->tune_gather = gather;
+                g.plan->tune_gather = gather ? 1 : 2;
                 g.plan->tune_rings = rings;
                 g.plan->tune_split = split;
                 double us = 0;
@@ -263,7 +263,7 @@ static int tune_group(zm_batch_t b, BatchGroup& g, const zm_request_t* reqs,
                 if (s != ZM_OK) return s;
                 if (us < best.us) best = TuneChoice{gather, rings, split, us};
             }
-    g.plan->tune_gather = best.gather;
+    g.plan->tune_gather = best.gather ? 1 : 2;
     g.plan->tune_rings = best.rings;
     g.plan->tune_split = best.split;
     cache[key] = best;

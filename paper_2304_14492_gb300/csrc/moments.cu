@@ -16,6 +16,7 @@ int launch_projection_tc(zm_plan_t p, const float* F, int batch, float* out, uns
 
 // ============================================================== K-b
 constexpr int KB_MAX_IMG = 128;
+constexpr long long GATHER_PDL_SAMPLES = 1ll << 18;
 
 struct KbParams {
     int n_rho, n_max, batch_total, b_off;
@@ -55,13 +56,39 @@ __device__ __forceinline__ float bilinear(const GeoImage& im, float X, float Y) 
     return fmaf(fy, bot - top, top);
 }
 
+// The same value, bit for bit, where the whole stencil is known to lie in an
+// image of less than 2^31 elements and 2^22 columns and rows: the floor is a
+// rounded-down addition of 2^23 (its low bits are the integer), one 32-bit
+// offset addresses all four pixels, and nothing is clamped or tested (22
+// instructions a sample where the general form takes about 50).
+__device__ __forceinline__ float bilinear_inside(const float* d, int pitch, float X, float Y) {
+    const float tx = __fadd_rd(X, 8388608.f), ty = __fadd_rd(Y, 8388608.f);
+    const float fx = X - (tx - 8388608.f), fy = Y - (ty - 8388608.f);
+    const int o = (__float_as_int(ty) - 0x4b000000) * pitch + (__float_as_int(tx) - 0x4b000000);
+    const float* r0 = d + o;
+    const float* r1 = r0 + pitch;
+    const float p00 = __ldg(r0), p01 = __ldg(r0 + 1), p10 = __ldg(r1), p11 = __ldg(r1 + 1);
+    const float top = fmaf(fx, p01 - p00, p00);
+    const float bot = fmaf(fx, p11 - p10, p10);
+    return fmaf(fy, bot - top, top);
+}
+
+// Every stencil of the ring of radius rad lies inside the image, with a pixel
+// to spare for the rounding of the sample coordinates (below 2^22 they are off
+// by less than that).
+__device__ __forceinline__ bool ring_inside(const GeoImage& im, float rad) {
+    return im.w < (1 << 22) && im.h < (1 << 22) && (long long)im.h * im.pitch < (1ll << 31) && im.cx - rad >= 1.f &&
+           im.cx + rad <= (float)(im.w - 3) && im.cy - rad >= 1.f && im.cy + rad <= (float)(im.h - 3);
+}
+
 // One CTA = R consecutive rings of one image at a time, one warp per ring
 // (R = blockDim/32); the grid is persistent and each CTA walks ring blocks
 // (image, block) after loading the FFT twiddles once.
-// Phase 1: the R x N samples into shared memory (bilinear gather; polar input
-// goes straight from global memory into the FFT registers).  Phase 2: per
-// warp, the N-point real FFT of its ring as an N/2-point complex FFT plus the
-// split
+// Phase 1: each warp's samples straight into its FFT registers: bilinear gather
+// (a lane takes the two angles of a packed point, so nothing passes through
+// shared memory and no barrier separates the warps), or the polar input.  Phase
+// 2: per warp, the N-point real FFT of its ring as an N/2-point complex FFT
+// plus the split
 //   F_m = (Z_m + conj Z_{M-m})/2 + e^{-2 pi i m/N} (Z_m - conj Z_{M-m})/(2i),
 // for m = 0..n_max.  Phase 3: F[m][b][re/im][i0..i0+R) written as segments.
 template <int LOGN, int MODE>
@@ -107,39 +134,72 @@ __global__ void __launch_bounds__(256, (LOGN >= 11 ? 2 : 4)) k_ring_spectra(cons
             }
         }
     };
+    griddep_wait();                // the images or polar samples are written, the spectra are free
+    griddep_launch();              // (the grid is resident at once)
     if (MODE == KB_POLAR && (int)blockIdx.x < n_items) load_ring(blockIdx.x);
+    bool ready = false;
     for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
         const int bl = item / n_rb;
         const int i0 = (item - bl * n_rb) * R;
         const int b = p.b_off + bl;
-        if (MODE != KB_POLAR) {
+        if (MODE == KB_RESAMPLE) {
             const GeoImage im = p.img[bl];
 #pragma unroll 4
             for (int idx = threadIdx.x; idx < R * N; idx += blockDim.x) {
                 const int r = idx >> LOGN, k = idx & (N - 1);
                 const int i = i0 + r;
-                float vv = 0.f;
                 if (i < n_rho) {
                     const float rad = im.r * __ldg(&p.rho32[i]);
                     const float2 c = __ldg(&p.cs[k]);
-                    vv = bilinear(im, fmaf(rad, c.x, im.cx), fmaf(-rad, c.y, im.cy));
-                    if (p.fhat_out) p.fhat_out[((size_t)b * n_rho + i) * N + k] = vv;
+                    p.fhat_out[((size_t)b * n_rho + i) * N + k] =
+                        bilinear(im, fmaf(rad, c.x, im.cx), fmaf(-rad, c.y, im.cy));
                 }
-                if (MODE != KB_RESAMPLE) rings[r * ROW + k] = vv;
+            }
+            continue;
+        }
+        if (MODE == KB_GATHER) {
+            const GeoImage& im = p.img[bl];
+            const int i = i0 + warp;
+#pragma unroll
+            for (int s = 0; s < FFT::Q; ++s) v[s] = make_float2(0.f, 0.f);
+            if (i < n_rho && lane < FFT::L) {
+                const float rad = im.r * __ldg(&p.rho32[i]);
+                const float4* cs2 = reinterpret_cast<const float4*>(p.cs);      // two angles
+                if (ring_inside(im, rad)) {
+                    const float* d = im.data;
+                    const int pitch = (int)im.pitch;
+                    const float cx = im.cx, cy = im.cy;
+#pragma unroll
+                    for (int s = 0; s < FFT::Q; ++s) {
+                        const float4 c = __ldg(&cs2[lane + FFT::L * s]);
+                        v[s].x = bilinear_inside(d, pitch, fmaf(rad, c.x, cx), fmaf(-rad, c.y, cy));
+                        v[s].y = bilinear_inside(d, pitch, fmaf(rad, c.z, cx), fmaf(-rad, c.w, cy));
+                    }
+                } else {
+#pragma unroll
+                    for (int s = 0; s < FFT::Q; ++s) {
+                        const float4 c = __ldg(&cs2[lane + FFT::L * s]);
+                        v[s].x = bilinear(im, fmaf(rad, c.x, im.cx), fmaf(-rad, c.y, im.cy));
+                        v[s].y = bilinear(im, fmaf(rad, c.z, im.cx), fmaf(-rad, c.w, im.cy));
+                    }
+                }
+                if (p.fhat_out) {
+                    float* dst = p.fhat_out + ((size_t)b * n_rho + i) * N;
+#pragma unroll
+                    for (int s = 0; s < FFT::Q; ++s) {
+                        dst[2 * (lane + FFT::L * s)] = v[s].x;
+                        dst[2 * (lane + FFT::L * s) + 1] = v[s].y;
+                    }
+                }
             }
         }
-        if (MODE == KB_RESAMPLE) continue;
-        __syncthreads();   // the twiddles (first block) and the gathered rings
+        if (!ready) {
+            __syncthreads();                           // the twiddles
+            ready = true;
+        }
 
         {
             float* row = rings + warp * ROW;
-            if (MODE != KB_POLAR) {
-                const float2* z = reinterpret_cast<const float2*>(row);
-#pragma unroll
-                for (int s = 0; s < FFT::Q; ++s)
-                    v[s] = (lane < FFT::L) ? z[lane + FFT::L * s] : make_float2(0.f, 0.f);
-                __syncwarp();
-            }
             float2* X = reinterpret_cast<float2*>(row);
             FFT::fwd(v, lane, twt, X);                 // the row doubles as the transpose buffer
             if (lane < FFT::L) {
@@ -164,10 +224,11 @@ __global__ void __launch_bounds__(256, (LOGN >= 11 ? 2 : 4)) k_ring_spectra(cons
         if (p.Fblk) {
             // R = 8 rings = one 16-byte row per (m, re/im): bf16 hi and lo halves
             const int ncol = 2 * p.batch_total;
+            // (re and im of an order are the halves of one 32-byte sector:
+            // adjacent threads, so that no sector is written in two pieces)
             for (int e = threadIdx.x; e < 2 * nm1; e += blockDim.x) {
-                const int c = e >= nm1 ? 1 : 0;
-                const int m = e - c * nm1;
-                const float* src = Fs + (size_t)e * 8;
+                const int c = e & 1, m = e >> 1;
+                const float* src = Fs + (size_t)(c * nm1 + m) * 8;
                 uint32_t h[4], l[4];
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {
@@ -406,8 +467,17 @@ static int launch_kb_t(const KbParams& kp, int R, int nb, cudaStream_t st) {
     k.nb = nb;
     const long long items = (long long)(kp.Fblk ? kp.n_chunks * (64 / R) : (kp.n_rho + R - 1) / R) * nb;
     const int grid = (int)std::min<long long>(items, (long long)per_sm * num_sms(dev));
-    k_ring_spectra<LOGN, MODE><<<grid, R * 32, smem, st>>>(kp);
-    ZM_LAUNCH_CHECK("k_ring_spectra");
+    // A gather of more than GATHER_PDL_SAMPLES is not launched early: it lives on
+    // L1, and CTAs that come in while the previous call's projection holds most
+    // of the SM's shared memory keep that split for their lifetime (16 images of
+    // 512 x 512 on a 256 x 256 grid, back to back: 27 us a call with the early
+    // launch, 18 without; 40 images of 1024 x 1024 on 512 x 256, FP32: 164 and 62).
+    if (MODE == KB_GATHER && (long long)nb * kp.n_rho * FFT::N > GATHER_PDL_SAMPLES) {
+        k_ring_spectra<LOGN, MODE><<<grid, R * 32, smem, st>>>(kp);
+        ZM_LAUNCH_CHECK("k_ring_spectra");
+        return ZM_OK;
+    }
+    ZM_LAUNCH_PDL("k_ring_spectra", (k_ring_spectra<LOGN, MODE>), dim3(grid), dim3(R * 32), smem, st, kp);
     return ZM_OK;
 }
 
@@ -496,12 +566,30 @@ static int launch_polar_fft(zm_plan_t p, const float* fhat, int b0, int nb, int 
     return ZM_OK;
 }
 
+// Where the gather kernel is the fastest of the three by default.  Its rings of
+// up to 256 angles leave a lane eight samples, whose loads are all in flight;
+// images come from L1 and L2, and no plan of tiles or stages stands before the
+// first pixel.  Measured per call, back to back (gather / fused or tiles, us,
+// bf16x3): 64 x 64 on 32 x 64, 1 image 5.6 / 6.6; 512 x 512 on 256 x 256, 4
+// images 10.9 / 16.0, 16 images 17.6 / 16.5, 40 images 30.6 / 33.1; 1024 x 1024
+// on 512 x 256, 40 images 56.7 / 66.9; 2160 x 2160 on 1080 x 256, 1 image 14.8 /
+// 20.0, 16 images 59.6 / 63.5.  At 512 angles (16 samples a lane) it holds up to
+// about 1.5 million samples a call: 512 x 512 on 256 x 512, 4 images 12.7 / 20.2,
+// 8 images 16.0 / 20.5, 16 images 24.1 / 21.1.  At 1024 it loses throughout
+// (2160 x 2160 on 1024 x 1024, 1 image 33 / 24, 16 images 382 / 87).  A plan told
+// to fuse or not to (ZM_FUSED), or to use a tensor-core transform, does that.
+static bool gather_by_default(zm_plan_t p, int batch) {
+    if (p->fused_mode != 0 || p->dft_mode > 0 || p->pdft_mode > 0) return false;
+    const long long samples = (long long)p->n_rho * p->n_theta;
+    return p->n_theta <= 256 || (p->n_theta == 512 && samples <= FUSED_AUTO_SAMPLES && samples * batch <= 3ll << 19);
+}
+
 // Ring spectra of a batch.  Polar input: FFT only.  Images: runs of one
 // geometry go through the tensor-core DFT kernel when the plan asks for it
 // (dft_mode, off by default) and the spectra are wanted as operand blocks
 // only (no polar samples out), else through the fused kernel when its fused_mode allows (resampling
 // and ring FFT in one pass, polar samples written only to the caller's
-// fhat_out);
+// fhat_out), unless the gather kernel is faster there (gather_by_default);
 // other runs of TMA-eligible images go through the tile resampler into the
 // polar buffer (the caller's fhat_out, else the plan workspace) and then the
 // ring FFT; the rest take the gather kernel.
@@ -510,10 +598,11 @@ int launch_spectra(zm_plan_t p, const zm_image_t* imgs, const float* fhat_in, in
     if (fhat_in) return launch_polar_fft(p, fhat_in, 0, batch, batch, F, Fblk, st);
     const bool fuse = p->fused_mode > 0 ||
                       (p->fused_mode == 0 && (long long)p->n_rho * p->n_theta <= FUSED_AUTO_SAMPLES);
-    const bool dft = Fblk && !fhat_out && !resample_only && !p->tune_gather && p->dft_mode > 0;
+    const bool gather = p->tune_gather == 1 || (p->tune_gather == 0 && !resample_only && gather_by_default(p, batch));
+    const bool dft = Fblk && !fhat_out && !resample_only && !gather && p->dft_mode > 0;
     auto use_dft = [&](int b) { return dft && dft_eligible(p, imgs[b]); };
-    auto use_fused = [&](int b) { return fuse && !resample_only && !p->tune_gather && fused_eligible(p, imgs[b]); };
-    auto use_tma = [&](int b) { return !p->tune_gather && tma_eligible(imgs[b]); };
+    auto use_fused = [&](int b) { return fuse && !resample_only && !gather && fused_eligible(p, imgs[b]); };
+    auto use_tma = [&](int b) { return !gather && tma_eligible(imgs[b]); };
     float* fh = fhat_out;
     int b = 0;
     while (b < batch) {
