@@ -91,8 +91,12 @@ __device__ __forceinline__ bool ring_inside(const GeoImage& im, float rad) {
 // plus the split
 //   F_m = (Z_m + conj Z_{M-m})/2 + e^{-2 pi i m/N} (Z_m - conj Z_{M-m})/(2i),
 // for m = 0..n_max.  Phase 3: F[m][b][re/im][i0..i0+R) written as segments.
+//
+// Residency: four CTAs per SM up to 512 angles.  At 1024 the 64 registers that
+// leaves cost the gather its loads in flight and, with 32 rings at once, its hits
+// in L1: 8 images of 2161 x 2161 on 1024 x 1024 took 248 us, with two CTAs 67.
 template <int LOGN, int MODE>
-__global__ void __launch_bounds__(256, (LOGN >= 11 ? 2 : 4)) k_ring_spectra(const __grid_constant__ KbParams p) {
+__global__ void __launch_bounds__(256, (LOGN >= 10 ? 2 : 4)) k_ring_spectra(const __grid_constant__ KbParams p) {
     using FFT = RingFFT<LOGN>;
     constexpr int N = FFT::N;
     constexpr int ROW = FFT::ROW_FLOATS;
@@ -502,7 +506,11 @@ static int pick_rings(zm_plan_t p, int batch) {
     if (p->tune_rings == 2 || p->tune_rings == 4 || p->tune_rings == 8) return p->tune_rings;
     int R = 8;
     const int want = 2 * num_sms(p->device);
-    while (R > 2 && ((p->n_rho + R - 1) / R) * batch < want) R >>= 1;
+    // two rings to a CTA spread small calls over the SMs; rings of 512 angles and
+    // more keep four (their twiddle tables are loaded by every CTA: one 2160 x
+    // 2160 image on 1024 x 1024, FP32, 20.8 us against 23.7 with two)
+    const int least = p->n_theta >= 512 ? 4 : 2;
+    while (R > least && ((p->n_rho + R - 1) / R) * batch < want) R >>= 1;
     return R;
 }
 
@@ -575,13 +583,20 @@ static int launch_polar_fft(zm_plan_t p, const float* fhat, int b0, int nb, int 
 // on 512 x 256, 40 images 56.7 / 66.9; 2160 x 2160 on 1080 x 256, 1 image 14.8 /
 // 20.0, 16 images 59.6 / 63.5.  At 512 angles (16 samples a lane) it holds up to
 // about 1.5 million samples a call: 512 x 512 on 256 x 512, 4 images 12.7 / 20.2,
-// 8 images 16.0 / 20.5, 16 images 24.1 / 21.1.  At 1024 it loses throughout
-// (2160 x 2160 on 1024 x 1024, 1 image 33 / 24, 16 images 382 / 87).  A plan told
-// to fuse or not to (ZM_FUSED), or to use a tensor-core transform, does that.
+// 8 images 16.0 / 20.5, 16 images 24.1 / 21.1 (grids of more than 2^17 samples
+// keep the tiles, whose lead at 8 images is as large).  At 1024 angles, with
+// operand blocks as output, up to the same number: 2160 x 2160 on 1024 x 1024,
+// 1 image 19.2 / 23.7, 4 images 42.7 / 34.8; 1024 x 1024 on 512 x 1024, 1 image
+// 26.8 / 30.9, 16 images 69 / 57.  With FP32 rows, whose ring FFT after the tiles
+// is cheaper, up to a third of it: 1024 x 1024 on 512 x 1024, 1 image 17.5 / 20.2;
+// 2160 x 2160 on 1024 x 1024, 1 image 20.8 / 18.6.  A plan told to fuse or not to
+// (ZM_FUSED), or to use a tensor-core transform, does that.
 static bool gather_by_default(zm_plan_t p, int batch) {
     if (p->fused_mode != 0 || p->dft_mode > 0 || p->pdft_mode > 0) return false;
     const long long samples = (long long)p->n_rho * p->n_theta;
-    return p->n_theta <= 256 || (p->n_theta == 512 && samples <= FUSED_AUTO_SAMPLES && samples * batch <= 3ll << 19);
+    if (p->n_theta <= 256) return true;
+    if (p->n_theta == 512) return samples <= FUSED_AUTO_SAMPLES && samples * batch <= 3ll << 19;
+    return p->n_theta == 1024 && samples * batch <= (blocked_projection(p) ? 3ll << 19 : 1ll << 19);
 }
 
 // Ring spectra of a batch.  Polar input: FFT only.  Images: runs of one
