@@ -9,7 +9,8 @@
 // request's prefix into its own output.  The whole sequence is captured once
 // into a CUDA graph and replayed while the request pointers stay the same;
 // the groups fork onto BATCH_BRANCHES side streams (balanced by pixel count),
-// so they become parallel branches of the graph and small groups overlap.
+// so they become parallel branches of the graph and small groups overlap; with
+// large groups the projections form a second phase (enqueue_batch).
 // Launch choices per group come from a small autotuner (timed candidates,
 // cached in a JSON file).
 #include <algorithm>
@@ -113,26 +114,51 @@ static void free_batch(zm_batch_t b) {
 
 namespace zm {
 
-// The whole batch from stream st: the groups fork onto the side streams (per
-// group resampling + ring FFT + projection into its buffer), join back on st,
-// then the prefix copies.
+// The whole batch from stream st: the groups fork onto the side streams, join
+// back on st, then the prefix copies.  Per group: resampling + ring FFT, then the
+// projection into its buffer.  Batches of small groups run the two in turn on
+// each branch; once a group gathers more samples than an early launch pays for
+// (GATHER_PDL_SAMPLES), all spectra come first and all projections after them: a
+// projection's shared memory would otherwise leave the gathers that share its SMs
+// little L1 (256 requests of 128 to 1024 pixels, bf16x3: 255 us a replay in turn,
+// 158 in two phases; all spectra on one stream 182.  12 requests: 40 and 44).
 static int enqueue_batch(zm_batch_t b, const zm_request_t* reqs, unsigned flags, cudaStream_t st) {
     std::vector<zm_image_t> imgs;
-    ZM_CUDA_TRY(cudaEventRecord(b->ev_fork, st));
-    for (int k = 0; k < BATCH_BRANCHES; ++k) ZM_CUDA_TRY(cudaStreamWaitEvent(b->side[k], b->ev_fork, 0));
-    for (size_t gi = 0; gi < b->groups.size(); ++gi) {
+    auto fork = [&]() -> int {
+        ZM_CUDA_TRY(cudaEventRecord(b->ev_fork, st));
+        for (int k = 0; k < BATCH_BRANCHES; ++k) ZM_CUDA_TRY(cudaStreamWaitEvent(b->side[k], b->ev_fork, 0));
+        return ZM_OK;
+    };
+    auto join = [&]() -> int {
+        for (int k = 0; k < BATCH_BRANCHES; ++k) {
+            ZM_CUDA_TRY(cudaEventRecord(b->ev_join[k], b->side[k]));
+            ZM_CUDA_TRY(cudaStreamWaitEvent(st, b->ev_join[k], 0));
+        }
+        return ZM_OK;
+    };
+    bool phases = false;
+    for (auto& g : b->groups)
+        phases = phases || (long long)g.n_rho * g.n_theta * (long long)g.members.size() > GATHER_PDL_SAMPLES;
+    int s = fork();
+    for (size_t gi = 0; gi < b->groups.size() && s == ZM_OK; ++gi) {
         auto& g = b->groups[gi];
         imgs.clear();
         for (int r : g.members) imgs.push_back(reqs[r].image);
         const int gb = (int)g.members.size();
-        const int s = launch_moments(g.plan, imgs.data(), nullptr, gb, g.out_buf, nullptr, flags,
-                                     b->side[b->branch[gi]]);
-        if (s != ZM_OK) return s;
+        cudaStream_t sg = b->side[b->branch[gi]];
+        s = launch_stage_spectra(g.plan, imgs.data(), nullptr, gb, nullptr, sg);
+        if (s == ZM_OK && !phases) s = launch_stage_project(g.plan, gb, g.out_buf, flags, sg, true);
     }
-    for (int k = 0; k < BATCH_BRANCHES; ++k) {
-        ZM_CUDA_TRY(cudaEventRecord(b->ev_join[k], b->side[k]));
-        ZM_CUDA_TRY(cudaStreamWaitEvent(st, b->ev_join[k], 0));
+    if (s == ZM_OK && phases) {
+        s = join();
+        if (s == ZM_OK) s = fork();
+        for (size_t gi = 0; gi < b->groups.size() && s == ZM_OK; ++gi) {
+            auto& g = b->groups[gi];
+            s = launch_stage_project(g.plan, (int)g.members.size(), g.out_buf, flags, b->side[gi % BATCH_BRANCHES], true);
+        }
     }
+    if (s == ZM_OK) s = join();
+    if (s != ZM_OK) return s;
     k_batch_copy<<<(unsigned)b->reqs.size(), 256, 0, st>>>(b->d_copy);
     ZM_LAUNCH_CHECK("k_batch_copy");
     return ZM_OK;
@@ -251,9 +277,16 @@ static int tune_group(zm_batch_t b, BatchGroup& g, const zm_request_t* reqs,
     for (int r : g.members) tma = tma && tma_eligible(reqs[r].image);
     TuneChoice best;
     best.us = 1e30;
-    for (int gather = 0; gather <= (tma ? 1 : 0); ++gather)
+    // up to 256 angles the gather kernel shares the device with other groups
+    // better than the staged ones, whatever each takes alone (256 requests: 158
+    // us a replay, 186 staged); rings and split matter only to FP32 spectra and to
+    // the split-K projection
+    const int first = g.plan->n_theta <= 256 ? 1 : 0;
+    const bool blocked = blocked_projection(g.plan);
+    for (int gather = first; gather <= (tma ? 1 : first); ++gather)
         for (int rings : {2, 4, 8})
             for (int split : {4, 8}) {
+                if (blocked && (rings < 8 || split < 8)) continue;
                 if (split > 4 && g.plan->prec == PREC_FP32) continue;      // no radial split there
                 g.plan->tune_gather = gather ? 1 : 2;
                 g.plan->tune_rings = rings;

@@ -16,7 +16,6 @@ int launch_projection_tc(zm_plan_t p, const float* F, int batch, float* out, uns
 
 // ============================================================== K-b
 constexpr int KB_MAX_IMG = 128;
-constexpr long long GATHER_PDL_SAMPLES = 1ll << 18;
 
 struct KbParams {
     int n_rho, n_max, batch_total, b_off;
@@ -693,7 +692,7 @@ int launch_stage_spectra(zm_plan_t p, const zm_image_t* imgs, const float* fhat_
 
 // Stage 2: the radial projection of the spectra stage 1 left in the workspace
 // (consume: no later call reads them, so the blocked form drops them from L2).
-int launch_stage_project(zm_plan_t p, int batch, float* out, unsigned flags, cudaStream_t st, bool consume = false) {
+int launch_stage_project(zm_plan_t p, int batch, float* out, unsigned flags, cudaStream_t st, bool consume) {
     if (blocked_projection(p))
         return launch_projection_blocked(p, (const uint8_t*)p->ws_Fblk.ptr, batch, out, flags, st, consume);
     return launch_projection(p, (const float*)p->ws_F.ptr, batch, out, flags, st);

@@ -235,6 +235,11 @@ int launch_projection_fp32(zm_plan_t p, const float* F, int batch, float* out, u
 // spectra, then the projection; bf16 plans take the blocked tensor-core path.
 int launch_moments(zm_plan_t p, const zm_image_t* imgs, const float* fhat_in, int batch, float* out,
                    float* fhat_out, unsigned flags, cudaStream_t st);
+// Its two stages: ring spectra into the plan's workspace, in the form the
+// projection reads, then the projection (consume: no later call reads them).
+int launch_stage_spectra(zm_plan_t p, const zm_image_t* imgs, const float* fhat_in, int batch, float* fhat_out,
+                         cudaStream_t st);
+int launch_stage_project(zm_plan_t p, int batch, float* out, unsigned flags, cudaStream_t st, bool consume = false);
 // Blocked tensor-core projection (project_tc.cu).
 int build_tc_blocks(zm_plan_t p);
 bool blocked_projection(zm_plan_t p);
@@ -306,6 +311,8 @@ inline GeoImage resolve(const zm_image_t& im) {
 int check_images(const zm_image_t* imgs, int batch);
 
 constexpr int RED_MAX_BLOCKS = 512;   // blocks (records) per image of the pixel and node reductions
+
+constexpr long long GATHER_PDL_SAMPLES = 1ll << 18;   // largest gather (samples) launched before its predecessor ends
 
 // Cartesian-tile resampling (resample_tiles.cu)
 bool tma_eligible(const zm_image_t& im);
