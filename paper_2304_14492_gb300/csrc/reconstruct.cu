@@ -173,13 +173,22 @@ k_recon_ifft(const float* __restrict__ G, const float2* __restrict__ tw, int n_m
     griddep_wait();                    // G (and the reference samples) are written, out is free
     griddep_launch();
     // persistent: the CTA takes ring blocks (b, rb) = item / n_rb, item mod n_rb
-    __shared__ int next_item;
+    __shared__ int next_item[2];
+    int turn = 0;
     const int n_rb = (n_rho + R - 1) / R;
     const int n_items = n_rb * batch;
     for (int item = blockIdx.x; item < n_items;) {
         const int b = item / n_rb, rb = item - b * n_rb;
         const int i0 = rb * R;
         // this block's G is one contiguous run of nm1 x 16 floats (g_index)
+        // the next item is claimed, and the reference rows are asked into L2,
+        // while this one is transformed
+        int claim = 0;
+        if (threadIdx.x == 0) claim = (int)gridDim.x + atomicAdd(&work[0], 1);
+        if (ERR && i0 + warp < n_rho) {
+            const char* rr = reinterpret_cast<const char*>(ref + ((size_t)b * n_rho + i0 + warp) * N);
+            for (int l = lane; l * 32 < N; l += 32) asm volatile("prefetch.global.L2 [%0];" ::"l"(rr + 128 * l));
+        }
         const float4* gb = reinterpret_cast<const float4*>(G + g_index(b, i0, 0, 0, n_rb, nm1));
         float* gsf = reinterpret_cast<float*>(Gs);
         for (int e = threadIdx.x; e < nm1 * 4; e += blockDim.x) {
@@ -266,10 +275,10 @@ k_recon_ifft(const float* __restrict__ G, const float2* __restrict__ tw, int n_m
             }
             if (lane == 0 && i < n_rho) part[(size_t)b * n_rho + i] = make_float4(sd, sf, mx, 0.f);
         }
-        if (threadIdx.x == 0) next_item = (int)gridDim.x + atomicAdd(&work[0], 1);
+        if (threadIdx.x == 0) next_item[turn] = claim;
         __syncthreads();   // Gs is refilled for the next ring block; next_item is set
-        item = next_item;
-        __syncthreads();   // every thread has read next_item before it is rewritten
+        item = next_item[turn];
+        turn ^= 1;         // rewritten only after the barrier above of the next block
     }
     // the last CTA out resets the counter (every CTA's last claim precedes its
     // arrival here)
@@ -457,78 +466,56 @@ __device__ __forceinline__ int last_node(const float* __restrict__ rho32, int n_
     return g;
 }
 
-// Polar reconstruction -> pixels.  A warp takes a 32 x 4 block of pixels as
-// four 8 x 4 tiles (a pixel of each tile per thread): the bilinear corners of
-// a compact tile fall on few 128-byte lines wherever it lies on the disk (a
-// 32 x 1 run along a radius touches a line per pixel), and stores still fill
-// whole 32-byte sectors.  The place of a pixel on the grid (square root,
-// division, atan2, node lookup: about 100 instructions) is computed once and
-// used for every image of the group; with it per image, one pixel per thread
-// and a ten-step search over the nodes, three 3840 x 2160 bands took 133 us,
-// now 69 us (both cold, serialised).  Bound by the L1 wavefronts of the corner
-// loads (62 % busy) and instruction issue (56 %).
-constexpr int PTC_TILES = 4, PTC_GROUP = 4;
+// Polar reconstruction -> pixels, one pixel per thread, a warp on an 8 x 4 tile:
+// the bilinear corners of a compact tile fall on few 128-byte lines wherever it
+// lies on the disk (a 32 x 1 run along a radius touches a line per pixel), and
+// stores still fill whole 32-byte sectors.  The place of a pixel on the grid
+// (square root, division, atan2, node lookup: about 100 instructions) is
+// computed once and used for every image of the group.  Bound by the latency
+// and the L1 wavefronts of the corner loads: with four pixels a thread and 24
+// warps per SM three 3840 x 2160 bands took 67 us, with one and 64 warps 59 (warm;
+// with the place per image and a ten-step search over the nodes 133, cold).
+constexpr int PTC_GROUP = 4;
 __global__ void __launch_bounds__(256) k_polar_to_cart(const __grid_constant__ CartParams p) {
     const CartGroup g = p.grp[blockIdx.z];
     const CanvasDesc c = p.cv[g.first];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int y = blockIdx.y * 32 + warp * 4 + (lane >> 3);
-    const int xb = blockIdx.x * 32 + (lane & 7);
-    if (y >= c.h) return;
+    const int x = blockIdx.x * 8 + (lane & 7);
+    if (y >= c.h || x >= c.w) return;
     const int n_rho = p.n_rho, N = p.n_theta;
-    // per pixel: the corners' offsets and the two fractions; o0 < 0: outside the disk
-    int o0[PTC_TILES], o1[PTC_TILES], dk[PTC_TILES];
-    float s[PTC_TILES], t[PTC_TILES];
-    bool any = false;
-#pragma unroll
-    for (int j = 0; j < PTC_TILES; ++j) {
-        o0[j] = -1;
-        float dx, dy;
-        const float rho = pixel_rho((float)(xb + 8 * j), (float)y, c.cx, c.cy, c.r, &dx, &dy);
-        if (rho <= 1.f && xb + 8 * j < c.w) {
-            float th = atan2f(dy, dx);
-            if (th < 0.f) th += kTwoPi;
-            const int lo = last_node(p.rho32, n_rho, p.gauss, rho);
-            const int i1 = min(lo + 1, n_rho - 1), i0 = max(lo, 0);
-            const float r0 = __ldg(&p.rho32[i0]), r1 = __ldg(&p.rho32[i1]);
-            const float span = r1 - r0;
-            const float tt = span > 0.f ? (rho - r0) / span : 0.f;
-            t[j] = fminf(fmaxf(tt, 0.f), 1.f);
-            const float v = th * (float)N / kTwoPi;
-            const float kf = floorf(v);
-            s[j] = v - kf;
-            const int k0 = ((int)kf) & (N - 1);
-            dk[j] = ((k0 + 1) & (N - 1)) - k0;
-            o0[j] = i0 * N + k0;
-            o1[j] = i1 * N + k0;
-            any = true;
-        }
+    // the corners' offsets (o0 < 0: outside the disk) and the two fractions
+    int o0 = -1, o1 = 0, dk = 0;
+    float s = 0.f, t = 0.f;
+    float dx, dy;
+    const float rho = pixel_rho((float)x, (float)y, c.cx, c.cy, c.r, &dx, &dy);
+    if (rho <= 1.f) {
+        float th = atan2f(dy, dx);
+        if (th < 0.f) th += kTwoPi;
+        const int lo = last_node(p.rho32, n_rho, p.gauss, rho);
+        const int i1 = min(lo + 1, n_rho - 1), i0 = max(lo, 0);
+        const float r0 = __ldg(&p.rho32[i0]), r1 = __ldg(&p.rho32[i1]);
+        const float span = r1 - r0;
+        t = fminf(fmaxf(span > 0.f ? (rho - r0) / span : 0.f, 0.f), 1.f);
+        const float v = th * (float)N / kTwoPi;
+        const float kf = floorf(v);
+        s = v - kf;
+        const int k0 = ((int)kf) & (N - 1);
+        dk = ((k0 + 1) & (N - 1)) - k0;
+        o0 = i0 * N + k0;
+        o1 = i1 * N + k0;
     }
     const size_t img = (size_t)n_rho * N;
     const float* pb = p.polar + (size_t)(p.b_off + g.first) * img;
+#pragma unroll 1
     for (int q = 0; q < g.count; ++q, pb += img) {
-        float a0[PTC_TILES], a1[PTC_TILES], b0[PTC_TILES], b1[PTC_TILES];
-        if (any) {
-#pragma unroll
-            for (int j = 0; j < PTC_TILES; ++j)
-                if (o0[j] >= 0) {
-                    a0[j] = __ldg(pb + o0[j]);
-                    a1[j] = __ldg(pb + o0[j] + dk[j]);
-                    b0[j] = __ldg(pb + o1[j]);
-                    b1[j] = __ldg(pb + o1[j] + dk[j]);
-                }
+        float val = 0.f;
+        if (o0 >= 0) {
+            const float a0 = __ldg(pb + o0), a1 = __ldg(pb + o0 + dk), b0 = __ldg(pb + o1), b1 = __ldg(pb + o1 + dk);
+            const float ra = fmaf(s, a1 - a0, a0), rb = fmaf(s, b1 - b0, b0);
+            val = fmaf(t, rb - ra, ra);
         }
-        float* row = p.cv[g.first + q].data + (size_t)y * p.cv[g.first + q].pitch;
-#pragma unroll
-        for (int j = 0; j < PTC_TILES; ++j) {
-            const int x = xb + 8 * j;
-            float val = 0.f;
-            if (o0[j] >= 0) {
-                const float ra = fmaf(s[j], a1[j] - a0[j], a0[j]), rb = fmaf(s[j], b1[j] - b0[j], b0[j]);
-                val = fmaf(t[j], rb - ra, ra);
-            }
-            if (x < c.w) row[x] = val;
-        }
+        p.cv[g.first + q].data[(size_t)y * p.cv[g.first + q].pitch + x] = val;
     }
 }
 
@@ -564,7 +551,7 @@ int launch_polar_to_cart(zm_plan_t p, const float* polar, int batch, const zm_ca
             else
                 cp.grp[groups++] = CartGroup{j, 1};
         }
-        k_polar_to_cart<<<dim3((wmax + 8 * PTC_TILES - 1) / (8 * PTC_TILES), (hmax + 31) / 32, groups), 256, 0, st>>>(cp);
+        k_polar_to_cart<<<dim3((wmax + 7) / 8, (hmax + 31) / 32, groups), 256, 0, st>>>(cp);
         ZM_LAUNCH_CHECK("k_polar_to_cart");
     }
     return ZM_OK;
