@@ -262,16 +262,20 @@ __global__ void __launch_bounds__(256, (LOGN >= 10 ? 2 : 4)) k_ring_spectra(cons
 }
 
 // Polar samples -> ring spectra as bf16 operand blocks (the blocked
-// projection's F), one item = a block of 8 rings of a group of 4 images (one
-// 8-column group of the blocks).  Warp w transforms ring i0 + w of the 4
-// images in turn (the next ring's samples are loaded as soon as the current
-// FFT has left the registers), splits each into F_m, m <= n_max, and stages
-// them as Fs[image][re/im][ring][m]; then 8 consecutive threads write one
-// full 128-byte line (8 columns x 8 rings) per order and half.
+// projection's F), one item = a block of 8 rings of IPI images (4: one 8-column
+// group of the blocks).  Warp w transforms ring i0 + w of the images in turn
+// (the next ring's samples are loaded as soon as the current FFT has left the
+// registers), splits each into F_m, m <= n_max, and stages them as
+// Fs[image][re/im][ring][m]; then 2 IPI consecutive threads write 32 IPI
+// consecutive bytes (a full line at 4) per order and half.
+// IPI is picked by launch_blk_t: small batches spread over the SMs and transform
+// no absent images (one 4K frame, tiles + FFT + projection: 23.9 us a call with
+// four, 19.4 with one), and the last round of items is not nearly empty (16 4K
+// frames are 512 items of four images on 456 slots: 87.3 us, with two 86.7).
 // Occupancy: three CTAs per SM at N = 1024 (shared memory, 69 KB each), so the
 // register bound is set for three (77 registers; at 64 for four the kernel was
 // 0.7 us per batch of 16 4K frames slower).
-template <int LOGN>
+template <int LOGN, int IPI>
 __global__ void __launch_bounds__(256, (LOGN >= 11 ? 2 : (LOGN == 10 ? 3 : 4)))
     k_ring_blk(const __grid_constant__ KbParams p) {
     using FFT = RingFFT<LOGN>;
@@ -282,13 +286,13 @@ __global__ void __launch_bounds__(256, (LOGN >= 11 ? 2 : (LOGN == 10 ? 3 : 4)))
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int n_rho = p.n_rho, n_max = p.n_max, nm1 = n_max + 1;
     float* rows = smem;                                       // [R][ROW]
-    float* Fs = smem + R * ROW;                               // [4][2][R][nm1]
-    float2* twt = reinterpret_cast<float2*>(smem + ((R * ROW + 64 * nm1 + 3) & ~3));
+    float* Fs = smem + R * ROW;                               // [IPI][2][R][nm1]
+    float2* twt = reinterpret_cast<float2*>(smem + ((R * ROW + 16 * IPI * nm1 + 3) & ~3));
     float2* twm = twt + FFT::TW_FLOAT2;                       // e^{-2 pi i m / N}, m <= n_max
     FFT::load_twiddles(twt, p.tw);
     for (int m = threadIdx.x; m <= n_max; m += blockDim.x) twm[m] = __ldg(&p.tw[m]);
     const int n_rb = p.n_chunks * (64 / R);
-    const int g0 = p.b_off >> 2, g1 = (p.b_off + p.nb - 1) >> 2;
+    const int g0 = p.b_off / IPI, g1 = (p.b_off + p.nb - 1) / IPI;
     const int ng = g1 - g0 + 1;
     const int n_items = n_rb * ng;
     const int ncol = 2 * p.batch_total;
@@ -298,7 +302,7 @@ __global__ void __launch_bounds__(256, (LOGN >= 11 ? 2 : (LOGN == 10 ? 3 : 4)))
     auto load_ring = [&](int item, int q) {
         const int gi = item / n_rb;
         const int i = (item - gi * n_rb) * R + warp;
-        const int b = (g0 + gi) * 4 + q;
+        const int b = (g0 + gi) * IPI + q;
         const bool live = lane < FFT::L && i < n_rho && in_run(b);
         const float* src = p.fhat_in + ((size_t)(live ? b : 0) * n_rho + (live ? i : 0)) * N;
         if ((reinterpret_cast<uintptr_t>(p.fhat_in) & 7) == 0) {
@@ -323,13 +327,13 @@ __global__ void __launch_bounds__(256, (LOGN >= 11 ? 2 : (LOGN == 10 ? 3 : 4)))
         const int gi = item / n_rb;
         const int rb = item - gi * n_rb;
         const int i0 = rb * R;
-        for (int q = 0; q < 4; ++q) {
+        for (int q = 0; q < IPI; ++q) {
             FFT::fwd(v, lane, twt, X);
             if constexpr (N >= 32) {
                 // the ring's samples are in the registers now: when they are the
                 // plan's scratch, their L2 lines are invalidated without a write
                 // back (every line of a ring row belongs to that ring alone)
-                const int b = (g0 + gi) * 4 + q;
+                const int b = (g0 + gi) * IPI + q;
                 if (p.discard_in && i0 + warp < n_rho && in_run(b)) {
                     const char* base = reinterpret_cast<const char*>(p.fhat_in + ((size_t)b * n_rho + i0 + warp) * N);
                     for (int l = lane; l < N / 32; l += 32)
@@ -342,7 +346,7 @@ __global__ void __launch_bounds__(256, (LOGN >= 11 ? 2 : (LOGN == 10 ? 3 : 4)))
             }
             __syncwarp();
             // the next ring into the registers while this one is split
-            if (q < 3) load_ring(item, q + 1);
+            if (q < IPI - 1) load_ring(item, q + 1);
             else if (item + (int)gridDim.x < n_items) load_ring(item + gridDim.x, 0);
             float* fre = Fs + ((q * 2 + 0) * R + warp) * nm1;
             float* fim = Fs + ((q * 2 + 1) * R + warp) * nm1;
@@ -361,10 +365,9 @@ __global__ void __launch_bounds__(256, (LOGN >= 11 ? 2 : (LOGN == 10 ? 3 : 4)))
         __syncthreads();
         // (m, column) -> one 16-byte row of 8 rings; columns of images outside
         // this run (or past the batch) are left to their own launch
-        for (int e = threadIdx.x; e < 8 * nm1; e += blockDim.x) {
-            const int col8 = e & 7, m = e >> 3;
-            const int q = col8 >> 1, c = col8 & 1;
-            const int b = (g0 + gi) * 4 + q;
+        for (int e = threadIdx.x; e < 2 * IPI * nm1; e += blockDim.x) {
+            const int m = e / (2 * IPI), q = (e % (2 * IPI)) >> 1, c = e & 1;
+            const int b = (g0 + gi) * IPI + q;
             if (!in_run(b)) continue;
             const float* src = Fs + ((q * 2 + c) * R) * nm1 + m;
             uint32_t h[4], l[4];
@@ -385,39 +388,61 @@ __global__ void __launch_bounds__(256, (LOGN >= 11 ? 2 : (LOGN == 10 ? 3 : 4)))
     }
 }
 
-template <int LOGN>
-static int launch_blk_t(const KbParams& kp, int nb, cudaStream_t st) {
+template <int LOGN, int IPI>
+static int blk_slots(const KbParams& kp, size_t* smem) {
     using FFT = RingFFT<LOGN>;
-    const size_t smem = sizeof(float) * (((size_t)8 * FFT::ROW_FLOATS + 64 * (kp.n_max + 1) + 3) & ~(size_t)3) +
-                        sizeof(float2) * ((size_t)FFT::TW_FLOAT2 + kp.n_max + 1);
+    *smem = sizeof(float) * (((size_t)8 * FFT::ROW_FLOATS + 16 * IPI * (kp.n_max + 1) + 3) & ~(size_t)3) +
+            sizeof(float2) * ((size_t)FFT::TW_FLOAT2 + kp.n_max + 1);
     int dev = 0;
     cudaGetDevice(&dev);
-    static size_t configured[64] = {0};
-    if (smem > 48 * 1024 && (dev >= 64 || smem > configured[dev])) {
-        ZM_CUDA_TRY(cudaFuncSetAttribute(k_ring_blk<LOGN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        if (dev < 64) configured[dev] = smem;
-    }
     static std::mutex mu;
-    static std::map<size_t, int> resident;
-    int per_sm = 0;
-    {
-        std::lock_guard<std::mutex> lk(mu);
-        auto it = resident.find(smem);
-        if (it != resident.end()) {
-            per_sm = it->second;
-        } else {
-            if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_ring_blk<LOGN>, 256, smem) != cudaSuccess ||
-                per_sm < 1)
-                per_sm = 1;
-            resident[smem] = per_sm;
+    static std::map<std::pair<int, size_t>, int> resident;     // (device, smem) -> CTAs on the device
+    static size_t configured[64] = {0};
+    std::lock_guard<std::mutex> lk(mu);
+    auto it = resident.find({dev, *smem});
+    if (it != resident.end()) return it->second;
+    if (*smem > 48 * 1024 && (dev >= 64 || *smem > configured[dev])) {
+        const cudaError_t e = cudaFuncSetAttribute(k_ring_blk<LOGN, IPI>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                   (int)*smem);
+        if (e != cudaSuccess) {
+            cuda_error(e, "cudaFuncSetAttribute(k_ring_blk)");
+            return 0;
         }
+        if (dev < 64) configured[dev] = *smem;
     }
+    int per_sm = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_ring_blk<LOGN, IPI>, 256, *smem) != cudaSuccess ||
+        per_sm < 1)
+        per_sm = 1;
+    return resident[{dev, *smem}] = per_sm * num_sms(dev);
+}
+
+template <int LOGN>
+static int launch_blk_t(const KbParams& kp, int nb, cudaStream_t st) {
     KbParams& k = const_cast<KbParams&>(kp);
     k.nb = nb;
-    const int ng = ((kp.b_off + nb - 1) >> 2) - (kp.b_off >> 2) + 1;
-    const long long items = (long long)kp.n_chunks * 8 * ng;
-    const int grid = (int)std::min<long long>(items, (long long)per_sm * num_sms(dev));
-    ZM_LAUNCH_PDL("k_ring_blk", k_ring_blk<LOGN>, dim3(grid), dim3(256), smem, st, kp);
+    size_t smem[3];
+    const int slots[3] = {blk_slots<LOGN, 1>(kp, &smem[0]), blk_slots<LOGN, 2>(kp, &smem[1]),
+                          blk_slots<LOGN, 4>(kp, &smem[2])};
+    if (!slots[0] || !slots[1] || !slots[2]) return ZM_ECUDA;
+    // rounds of items (past the first, the CTAs drift apart: half a round of
+    // tail) times an item's rings per warp, its barriers and stores counted as
+    // half a ring.  Items of four stay where they fill the device well past once
+    // (24 images: within 3 % either way), and a pair of images stays together
+    // (its 64-byte pieces: 512 x 256 grid 13.5 us a call, apart 16.6)
+    int best = 2;
+    long long items[3];
+    double cost[3];
+    for (int j = 2; j >= 0; --j) {
+        const int ipi = 1 << j;
+        items[j] = (long long)kp.n_chunks * 8 * ((kp.b_off + nb - 1) / ipi - kp.b_off / ipi + 1);
+        const double rounds = items[j] > slots[j] ? (double)items[j] / slots[j] + 0.5 : 1.0;
+        cost[j] = rounds * (ipi + 0.5);
+        if (items[2] < 1.25 * slots[2] && !(j == 0 && nb == 2) && cost[j] < cost[best]) best = j;
+    }
+    const int grid = (int)std::min<long long>(items[best], slots[best]);
+    auto kernel = best == 0 ? k_ring_blk<LOGN, 1> : (best == 1 ? k_ring_blk<LOGN, 2> : k_ring_blk<LOGN, 4>);
+    ZM_LAUNCH_PDL("k_ring_blk", kernel, dim3(grid), dim3(256), smem[best], st, kp);
     return ZM_OK;
 }
 
