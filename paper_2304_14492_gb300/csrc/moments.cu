@@ -601,8 +601,9 @@ static int launch_polar_fft(zm_plan_t p, const float* fhat, int b0, int nb, int 
 // Where the gather kernel is the fastest of the three by default.  Its rings of
 // up to 256 angles leave a lane eight samples, whose loads are all in flight;
 // images come from L1 and L2, and no plan of tiles or stages stands before the
-// first pixel.  (At 256 angles and about a million samples the staged kernel is
-// ahead by 5 to 10 %.)  Measured per call, back to back (gather / fused or tiles, us,
+// first pixel.  (At 256 angles and about a million samples in small grids the
+// staged kernel is ahead by 5 to 10 %; against the tiles of larger grids the
+// gather leads: 2160 x 2160 on 1080 x 256, 4 images 21.4 / 27.6.)  Measured per call, back to back (gather / fused or tiles, us,
 // bf16x3): 64 x 64 on 32 x 64, 1 image 5.6 / 6.6; 512 x 512 on 256 x 256, 4
 // images 10.9 / 16.0, 16 images 17.6 / 16.5, 40 images 30.6 / 33.1; 1024 x 1024
 // on 512 x 256, 40 images 56.7 / 66.9; 2160 x 2160 on 1080 x 256, 1 image 14.8 /
@@ -620,7 +621,8 @@ static bool gather_by_default(zm_plan_t p, int batch) {
     if (p->fused_mode != 0 || p->dft_mode > 0 || p->pdft_mode > 0) return false;
     const long long samples = (long long)p->n_rho * p->n_theta;
     if (p->n_theta < 256) return true;
-    if (p->n_theta == 256) return samples * batch <= 1ll << 19 || samples * batch > 3ll << 19;
+    if (p->n_theta == 256)
+        return samples > FUSED_AUTO_SAMPLES || samples * batch <= 1ll << 19 || samples * batch > 3ll << 19;
     if (p->n_theta == 512) return samples <= FUSED_AUTO_SAMPLES && samples * batch <= 3ll << 19;
     return p->n_theta == 1024 && samples * batch <= (blocked_projection(p) ? 3ll << 19 : 1ll << 19);
 }

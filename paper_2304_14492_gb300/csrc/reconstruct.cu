@@ -659,11 +659,17 @@ __global__ void __launch_bounds__(RED_THREADS, RED_PER_SM) k_reduce(const __grid
     const CanvasDesc& t = p.tst[bl];
     const int rows = MODE == RED_POLAR_ERRORS ? (p.n_nodes + RED_SEG - 1) / RED_SEG : c.h;
     const long long stride = gridDim.x * RED_WARPS;
+    bool waited = false;
     for (long long y0 = blockIdx.x * RED_WARPS + w; y0 < rows; y0 += 32 * stride) {
         // lane l: the span of the l-th of this warp's next 32 rows
         int sa = 0, sb = 0;
         if (MODE != RED_POLAR_ERRORS) {
             if (y0 + l * stride < rows) disk_span(c, (int)(y0 + l * stride), &sa, &sb);
+        }
+        if (!waited) {                 // the images are written, the records are free
+            griddep_wait();
+            griddep_launch();
+            waited = true;
         }
         for (int q = 0; q < 32 && y0 + q * stride < rows; ++q) {
             const int y = (int)(y0 + q * stride);
@@ -715,6 +721,10 @@ __global__ void __launch_bounds__(RED_THREADS, RED_PER_SM) k_reduce(const __grid
                     }
             }
         }
+    }
+    if (!waited) {                     // a warp without rows
+        griddep_wait();
+        griddep_launch();
     }
     __shared__ float sh[3][RED_WARPS];
     __shared__ long long shc[RED_WARPS];
@@ -893,8 +903,7 @@ static int run_reduce(zm_plan_t p, const zm_image_t* ref, const zm_image_t* tst,
         }
         const int blocks = row_blocks(p, rows, nb);
         rp.part = (double*)p->ws_red.ptr;         // each launch finishes its own images
-        k_reduce<MODE><<<dim3(blocks, nb), RED_THREADS, 0, st>>>(rp);
-        ZM_LAUNCH_CHECK("k_reduce");
+        ZM_LAUNCH_PDL("k_reduce", k_reduce<MODE>, dim3(blocks, nb), dim3(RED_THREADS), 0, st, rp);
     }
     return ZM_OK;
 }
@@ -923,6 +932,8 @@ __global__ void __launch_bounds__(RED_THREADS) k_minmax_apply(const __grid_const
     const CanvasDesc& c = p.cv[blockIdx.y];
     const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
     const int b = p.b_off + blockIdx.y;
+    griddep_wait();                    // the canvases and their min / max are written
+    griddep_launch();
     const float gmin = p.mm[2 * b], gmax = p.mm[2 * b + 1];
     const float lo = p.target[2 * b], hi = p.target[2 * b + 1];
     const float scale = gmax > gmin ? (hi - lo) / (gmax - gmin) : 0.f;
@@ -970,8 +981,7 @@ int launch_minmax_normalize(zm_plan_t p, const zm_canvas_t* cv, int batch, const
             np.cv[j] = resolve_canvas(cv[b0 + j]);
             hmax = std::max(hmax, np.cv[j].h);
         }
-        k_minmax_apply<<<dim3(row_blocks(p, hmax, nb), nb), RED_THREADS, 0, st>>>(np);
-        ZM_LAUNCH_CHECK("k_minmax_apply");
+        ZM_LAUNCH_PDL("k_minmax_apply", k_minmax_apply, dim3(row_blocks(p, hmax, nb), nb), dim3(RED_THREADS), 0, st, np);
     }
     return ZM_OK;
 }
