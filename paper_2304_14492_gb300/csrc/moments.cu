@@ -20,7 +20,7 @@ constexpr int KB_MAX_IMG = 128;
 struct KbParams {
     int n_rho, n_max, batch_total, b_off;
     int nb;                // images in this launch
-    uint8_t* Fblk;         // bf16 hi / lo operand blocks of F (R = 8), or NULL
+    uint8_t* Fblk;         // bf16 hi / lo operand blocks of F (R = 8 or 4), or NULL
     size_t fblk_half;      // bytes of one half
     int n_chunks;          // 64-node chunks of the radial index
     const float* rho32;    // [n_rho]
@@ -225,25 +225,32 @@ __global__ void __launch_bounds__(256, (LOGN >= 10 ? 2 : 4)) k_ring_spectra(cons
         __syncthreads();
         const int nm1 = n_max + 1;
         if (p.Fblk) {
-            // R = 8 rings = one 16-byte row per (m, re/im): bf16 hi and lo halves
+            // 8 rings = one 16-byte row per (m, re/im): bf16 hi and lo halves
+            // (R = 4: half a row)
             const int ncol = 2 * p.batch_total;
             // (re and im of an order are the halves of one 32-byte sector:
             // adjacent threads, so that no sector is written in two pieces)
             for (int e = threadIdx.x; e < 2 * nm1; e += blockDim.x) {
                 const int c = e & 1, m = e >> 1;
-                const float* src = Fs + (size_t)(c * nm1 + m) * 8;
+                const float* src = Fs + (size_t)(c * nm1 + m) * R;
                 uint32_t h[4], l[4];
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {
+                    if (2 * q >= R) break;
                     const __nv_bfloat16 h0 = __float2bfloat16_rn(src[2 * q]), h1 = __float2bfloat16_rn(src[2 * q + 1]);
                     const __nv_bfloat16 l0 = __float2bfloat16_rn(src[2 * q] - __bfloat162float(h0));
                     const __nv_bfloat16 l1 = __float2bfloat16_rn(src[2 * q + 1] - __bfloat162float(h1));
                     h[q] = __bfloat16_as_ushort(h0) | ((uint32_t)__bfloat16_as_ushort(h1) << 16);
                     l[q] = __bfloat16_as_ushort(l0) | ((uint32_t)__bfloat16_as_ushort(l1) << 16);
                 }
-                const size_t o = fblk_row(m, i0, 2 * b + c, p.n_chunks, ncol);
-                *reinterpret_cast<uint4*>(p.Fblk + o) = make_uint4(h[0], h[1], h[2], h[3]);
-                *reinterpret_cast<uint4*>(p.Fblk + p.fblk_half + o) = make_uint4(l[0], l[1], l[2], l[3]);
+                const size_t o = fblk_row(m, i0 & ~7, 2 * b + c, p.n_chunks, ncol) + 2 * (i0 & 7);
+                if (R == 8) {
+                    *reinterpret_cast<uint4*>(p.Fblk + o) = make_uint4(h[0], h[1], h[2], h[3]);
+                    *reinterpret_cast<uint4*>(p.Fblk + p.fblk_half + o) = make_uint4(l[0], l[1], l[2], l[3]);
+                } else {
+                    *reinterpret_cast<uint2*>(p.Fblk + o) = make_uint2(h[0], h[1]);
+                    *reinterpret_cast<uint2*>(p.Fblk + p.fblk_half + o) = make_uint2(l[0], l[1]);
+                }
             }
         } else {
             const int lgR = __ffs(R) - 1;                 // R is a power of two
@@ -542,7 +549,13 @@ static int pick_rings(zm_plan_t p, int batch) {
 // when fhat_out is set, the polar samples.
 static int launch_gather(zm_plan_t p, const zm_image_t* imgs, int b0, int nb, int batch, float* F, float* fhat_out,
                          bool resample_only, uint8_t* Fblk, cudaStream_t st) {
-    const int R = Fblk ? 8 : pick_rings(p, batch);
+    // operand blocks take whole rows of 8 rings; calls of few blocks are spread
+    // over twice the CTAs instead (us a call with 8 / 4 rings: one 256 x 256 image
+    // on 128 x 256 8.3 / 7.5, on 64 x 1024 11.7 / 9.3; one 1024 x 1024 on 512 x
+    // 1024 19.2 / 16.1; beyond, the half rows cost more: four 256 x 256 images on
+    // 128 x 128 7.1 / 7.4)
+    const long long blocks = 8ll * p->n_chunks * batch;
+    const int R = Fblk ? (blocks <= (p->n_theta >= 1024 ? 64 : 32) ? 4 : 8) : pick_rings(p, batch);
     static thread_local KbParams kp;
     kp.Fblk = resample_only ? nullptr : Fblk;
     kp.fblk_half = fblk_half_bytes(p->n_max, p->n_chunks, 2 * batch);
@@ -603,11 +616,11 @@ static int launch_polar_fft(zm_plan_t p, const float* fhat, int b0, int nb, int 
 // images come from L1 and L2, and no plan of tiles or stages stands before the
 // first pixel.  (At 256 angles and about a million samples in small grids the
 // staged kernel is ahead by 5 to 10 %; against the tiles of larger grids the
-// gather leads: 2160 x 2160 on 1080 x 256, 4 images 21.4 / 27.6.)  Measured per call, back to back (gather / fused or tiles, us,
-// bf16x3): 64 x 64 on 32 x 64, 1 image 5.6 / 6.6; 512 x 512 on 256 x 256, 4
-// images 10.9 / 16.0, 16 images 17.6 / 16.5, 40 images 30.6 / 33.1; 1024 x 1024
-// on 512 x 256, 40 images 56.7 / 66.9; 2160 x 2160 on 1080 x 256, 1 image 14.8 /
-// 20.0, 16 images 59.6 / 63.5.  At 512 angles (16 samples a lane) it holds up to
+// gather leads: 2160 x 2160 on 1080 x 256, 4 images 21.4 / 27.6.)  Measured per
+// call, back to back (gather / fused or tiles, us, bf16x3): 64 x 64 on 32 x 64, 1
+// image 5.5 / 6.6; 512 x 512 on 256 x 256, 4 images 9.8 / 16.0, 16 images 17.6 /
+// 16.5, 40 images 30.6 / 33.1; 1024 x 1024 on 512 x 256, 40 images 56.4 / 66.9;
+// 2160 x 2160 on 1080 x 256, 1 image 14.4 / 20.0, 16 images 59.6 / 63.5.  At 512 angles (16 samples a lane) it holds up to
 // about 1.5 million samples a call: 512 x 512 on 256 x 512, 4 images 12.7 / 20.2,
 // 8 images 16.0 / 20.5, 16 images 24.1 / 21.1 (grids of more than 2^17 samples
 // keep the tiles, whose lead at 8 images is as large).  At 1024 angles, with
