@@ -9,7 +9,7 @@
 //
 // One CTA = one m, 128 image columns (the MMA's M), all K_m orders (the MMA's
 // N, padded to a multiple of 16) and one slice of the radial index i (the
-// reduction, split over CTAs and summed by k_project_reduce).  Per 64-wide
+// reduction, split over CTAs and summed by k_project_reduce_tc).  Per 64-wide
 // chunk of i: the 128 threads load F (fp32), split it and store both halves in
 // the K-major, no-swizzle canonical layout (8-row x 16-byte core matrices;
 // core matrices adjacent in K are LBO = 128 B apart, 8-row groups SBO = 1024 B

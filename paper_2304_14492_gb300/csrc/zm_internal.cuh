@@ -200,9 +200,10 @@ struct zm_plan_s {
     int tune_gather = 0;        // 1: the gather kernel even where images could be staged; 2: staged where they can be
     int tune_rings = 0;         // rings per CTA of the ring-FFT kernels (2, 4 or 8)
     int tune_split = 0;         // CTAs per SM aimed at by the projection's radial split
-    // resampling fused with the ring FFT (ring_fused.cu): 0 = for images of at
-    // most FUSED_AUTO_SAMPLES polar samples (where it measured faster than
-    // the tile resampler + ring FFT), 1 = wherever it applies, -1 = never;
+    // resampling fused with the ring FFT from staged rows (ring_fused.cu): 0 =
+    // for images of at most FUSED_AUTO_SAMPLES polar samples (where it measured
+    // faster than the tile resampler + ring FFT) in calls that do not gather
+    // (gather_by_default), 1 = wherever it applies, -1 = never;
     // set from the environment variable ZM_FUSED ("1" / "0") at plan creation
     int fused_mode = 0;
     int staged_batch = 0;       // images whose spectra zm_stage_spectra left in the workspace
