@@ -22,6 +22,7 @@
 
 #include <algorithm>
 
+#include "column_scale.cuh"
 #include "tc_common.cuh"
 #include "zm_internal.cuh"
 
@@ -46,15 +47,6 @@ struct TcParams {
     float a_scale;           // A halves hold A * a_scale
 };
 
-// Power-of-two scale putting a column's largest |F| just below 2^14, so the
-// fp16 halves neither overflow nor lose the low part to subnormals.
-__device__ __forceinline__ float column_scale(float mx) {
-    if (!(mx > 0.f) || !isfinite(mx)) return 1.f;
-    int e;
-    frexpf(mx, &e);
-    return ldexpf(1.f, 14 - e);
-}
-
 // fp16: the scales of this CTA's columns over its own slice [ib, ie) of the
 // radius, eight threads a column.  A slice's partial sums leave the kernel
 // unscaled, so every slice can take its own scale; maxima over all m and nodes
@@ -62,7 +54,7 @@ __device__ __forceinline__ float column_scale(float mx) {
 // 1001 crops at n_max 80), here they are a second look at data the CTA loads
 // anyway.
 __device__ __forceinline__ void slice_scales(const float* Fm, int vrows, int col0, int n_rho, int ib, int ie, bool vec,
-                                             float* cscale) {
+                                             float a_scale, float* cscale) {
     const int g = threadIdx.x & 7;
     for (int r0 = 0; r0 < vrows; r0 += TC_THREADS / 8) {
         const int row = r0 + (threadIdx.x >> 3);
@@ -81,7 +73,7 @@ __device__ __forceinline__ void slice_scales(const float* Fm, int vrows, int col
             }
         }
         for (int o = 4; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-        if (g == 0 && row < vrows) cscale[row] = column_scale(mx);
+        if (g == 0 && row < vrows) cscale[row] = column_scale(mx, a_scale);
     }
 }
 
@@ -132,7 +124,7 @@ __global__ void __launch_bounds__(TC_THREADS) k_project_tc(const __grid_constant
     const bool fvec = (p.n_rho & 3) == 0 && (reinterpret_cast<uintptr_t>(p.F) & 15) == 0;
     const bool avec = (p.n_rho & 7) == 0;
     if (p.fp16) {
-        slice_scales(Fm, vrows, col0, p.n_rho, ib, ie, fvec, cscale);
+        slice_scales(Fm, vrows, col0, p.n_rho, ib, ie, fvec, p.a_scale, cscale);
         __syncthreads();
     }
     const unsigned long long t0 = global_ns();
