@@ -842,7 +842,7 @@ extern "C" int zm_plan_reserve(zm_plan_t plan, int batch) {
     if (s == ZM_OK && plan->prec != PREC_FP32) s = plan->ws_part.grow(sizeof(float) * S * plan->P * 2 * nb);
     if (s == ZM_OK) s = plan->ws_G.grow(sizeof(float) * g_floats(batch, plan->n_rho, plan->n_max));
     // reductions: a record per block of an image (pixel errors) or per ring (fused errors)
-    const size_t rec = std::max<size_t>(RED_MAX_BLOCKS, (size_t)plan->n_rho);
+    const size_t rec = std::max<size_t>(RED_MAX_PARTS, (size_t)plan->n_rho);
     if (s == ZM_OK) s = plan->ws_red.grow(sizeof(double) * nb * rec * 4);
     if (s == ZM_OK) s = plan->ws_scale.grow(sizeof(float) * 2 * nb);
     if (s == ZM_OK && blocked_projection(plan))

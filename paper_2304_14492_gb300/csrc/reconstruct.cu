@@ -12,7 +12,6 @@
 
 namespace zm {
 
-constexpr int KD_MAX_IMG = 128;
 constexpr float kTwoPi = 6.28318530717958647692f;
 
 // ============================================================== radial part
@@ -562,15 +561,17 @@ constexpr int RED_THREADS = 256;
 constexpr int RED_WARPS = RED_THREADS / 32;
 constexpr int RED_PER_SM = 6;            // resident blocks per SM the registers allow
 constexpr int RED_SEG = 2048;            // polar nodes a warp takes at a time
+constexpr int RED_PARTS = 32;            // parts a block keeps in shared memory
 
 enum { RED_DISK_ERRORS = 0, RED_POLAR_ERRORS = 1, RED_DISK_MINMAX = 2 };
 
 struct RedParams {
-    int n_nodes, b_off, nb;
+    int n_nodes, b_off;
+    int share;                // blocks an image may take (part_blocks)
     const float* fhat;        // polar errors
     const float* frec;
-    double* part;             // [image of the launch][gridDim.x][4]
-    int* done;                // blocks finished, 0 between launches
+    double* part;             // [image of the launch][RED_MAX_PARTS][4]
+    int* done;                // [image of the launch] blocks finished, 0 between launches
     double* out;              // error modes: [batch][4]
     float* mm;                // min / max: [batch][2]
     CanvasDesc ref[KD_MAX_IMG];
@@ -627,16 +628,37 @@ __device__ __forceinline__ float warp_min(float v) {
     return v;
 }
 
+// Parts an image of so many rows is summed in, one record each: a row per warp up
+// to RED_MAX_PARTS parts.  The image's own rows alone decide, so that the order of
+// its sums, and with it every bit of them, does not depend on the images it shares
+// a launch with.
+__host__ __device__ __forceinline__ int row_parts(int rows) {
+    const int n = (rows + RED_WARPS - 1) / RED_WARPS;
+    return n < 1 ? 1 : (n < RED_MAX_PARTS ? n : RED_MAX_PARTS);
+}
+
+// Blocks that take an image's parts in turn: all that are resident at once, shared
+// by the images of the launch (a block more for every part costs its own latency:
+// 8 images of 4000 x 64, 25 us against 11), with RED_PARTS parts at most for one.
+__host__ __device__ __forceinline__ int part_blocks(int parts, int share) {
+    const int least = (parts + RED_PARTS - 1) / RED_PARTS;
+    const int n = share > least ? share : least;
+    return n < parts ? n : parts;
+}
+
 // Sums over the disk's pixels or the polar nodes: (sum (f - g)^2, sum f^2,
 // max f, count) for the error modes, (min, max) for the min / max mode.  A warp
 // takes whole rows (runs of RED_SEG nodes), of which it reads only the disk's
 // columns, four 16-byte loads in flight per lane, with no test per pixel: bound
-// by memory.  Float partials per thread, one double record per block; the last
-// block to finish adds an image's records in a fixed order and writes the
-// result, so there is no second launch.  Three 3840 x 2160 bands: min / max
-// 151 + 5 us -> 19 us, errors 166 + 5 us -> 28 us (both cold, serialised; 44
-// and 88 MB read).  Before, 64 blocks an image tested every pixel with a
-// square root and a division and had one load in flight.
+// by memory.  Two 16-byte words are summed as a tree before they join a lane's
+// FP32 partial (a row of 3840 is 15 steps of it, pixel by pixel it was 120), each
+// part (row_parts) is a double record, and an image's last block to finish adds its
+// records in a fixed order and writes the result, so there is no second launch.
+// Three 3840 x 2160 bands: min / max 151 + 5 us -> 19 us, errors 166 + 5 us -> 28 us
+// (both cold, serialised; 44 and 88 MB read).  Before, 64 blocks an image tested
+// every pixel with a square root and a division and had one load in flight.  A flat
+// 4K image in a launch of 128 is off by 1.2e-7 (by lanes that ran on over an
+// image's share of the device's blocks 2.0e-5; worst of three, emulated).
 template <int MODE>
 __global__ void __launch_bounds__(RED_THREADS, RED_PER_SM) k_reduce(const __grid_constant__ RedParams p) {
     constexpr int U = MODE == RED_DISK_MINMAX ? 4 : 2;     // 16-byte loads in flight per lane and image
@@ -655,24 +677,47 @@ __global__ void __launch_bounds__(RED_THREADS, RED_PER_SM) k_reduce(const __grid
         }
         mx = fmaxf(mx, f);
     };
+    // the sums of a 16-byte word, (f - g)^2 and f^2, as trees
+    auto word = [&](const float4& f, const float4& g, float* d2, float* f2) {
+        const float dx = f.x - g.x, dy = f.y - g.y, dz = f.z - g.z, dw = f.w - g.w;
+        *d2 = fmaf(dy, dy, dx * dx) + fmaf(dw, dw, dz * dz);
+        *f2 = fmaf(f.y, f.y, f.x * f.x) + fmaf(f.w, f.w, f.z * f.z);
+        mx = fmaxf(fmaxf(mx, fmaxf(f.x, f.y)), fmaxf(f.z, f.w));
+    };
     const CanvasDesc& c = p.ref[bl];
     const CanvasDesc& t = p.tst[bl];
     const int rows = MODE == RED_POLAR_ERRORS ? (p.n_nodes + RED_SEG - 1) / RED_SEG : c.h;
-    const long long stride = gridDim.x * RED_WARPS;
-    bool waited = false;
-    for (long long y0 = blockIdx.x * RED_WARPS + w; y0 < rows; y0 += 32 * stride) {
+    // (minima and maxima are the same in any order: no more parts than blocks)
+    const int parts = MODE == RED_DISK_MINMAX ? min(row_parts(rows), p.share) : row_parts(rows);
+    const int blocks = part_blocks(parts, p.share);
+    if ((int)blockIdx.x >= blocks) return;       // the launch holds a taller image
+    // this block takes the parts blockIdx.x, + blocks, ..; a warp has the rows
+    // part * RED_WARPS + w, + parts * RED_WARPS, .. of each
+    const int mine = (parts - 1 - (int)blockIdx.x) / blocks + 1;
+    const int per = (rows + parts * RED_WARPS - 1) / (parts * RED_WARPS);
+    auto row_of = [&](int q) {
+        const int v = q / per;
+        return ((long long)blockIdx.x + (long long)v * blocks) * RED_WARPS + w + (long long)(q - v * per) * parts * RED_WARPS;
+    };
+    __shared__ float sh[2][RED_PARTS][RED_WARPS];
+    __shared__ float shm[2][RED_WARPS];
+    __shared__ long long shc[RED_WARPS];
+    __shared__ int is_last;
+    int left = per, part = 0;                    // rows left of the part in hand
+    const int total = mine * per;
+    long long first = blockIdx.x * RED_WARPS + w, yl = first;
+    for (int q0 = 0; q0 < total; q0 += 32) {
         // lane l: the span of the l-th of this warp's next 32 rows
         int sa = 0, sb = 0;
         if (MODE != RED_POLAR_ERRORS) {
-            if (y0 + l * stride < rows) disk_span(c, (int)(y0 + l * stride), &sa, &sb);
+            if (q0 + l < total && row_of(q0 + l) < rows) disk_span(c, (int)row_of(q0 + l), &sa, &sb);
         }
-        if (!waited) {                 // the images are written, the records are free
+        if (q0 == 0) {                           // the images are written, the records are free
             griddep_wait();
             griddep_launch();
-            waited = true;
         }
-        for (int q = 0; q < 32 && y0 + q * stride < rows; ++q) {
-            const int y = (int)(y0 + q * stride);
+        for (int q = 0; q < 32 && q0 + q < total; ++q) {
+            const int y = (int)yl;               // = row_of(q0 + q)
             int xa, xb;
             const float *f, *g;
             if (MODE == RED_POLAR_ERRORS) {
@@ -686,129 +731,153 @@ __global__ void __launch_bounds__(RED_THREADS, RED_PER_SM) k_reduce(const __grid
                 f = c.data + (long long)y * c.pitch;
                 g = MODE == RED_DISK_ERRORS ? t.data + (long long)y * t.pitch : f;
             }
-            if (xa >= xb) continue;
-            cnt += xb - xa;
-            int va, vb;
-            vector_span(f, xa, xb, &va, &vb);
-            // the columns outside the aligned middle: lane by lane
-            for (int x = xa + l; x < va; x += 32) add(__ldg(f + x), MODE != RED_DISK_MINMAX ? __ldg(g + x) : 0.f);
-            for (int x = vb + l; x < xb; x += 32) add(__ldg(f + x), MODE != RED_DISK_MINMAX ? __ldg(g + x) : 0.f);
-            const bool gvec = ((reinterpret_cast<uintptr_t>(g + va)) & 15) == 0;
-            const int nv = (vb - va) >> 2;
-            for (int v0 = l; v0 < nv; v0 += 32 * U) {
-                float4 fv[U], gv[U];
-#pragma unroll
-                for (int u = 0; u < U; ++u)
-                    if (v0 + 32 * u < nv) fv[u] = __ldg(reinterpret_cast<const float4*>(f + va) + v0 + 32 * u);
-#pragma unroll
-                for (int u = 0; u < U; ++u) gv[u] = make_float4(0.f, 0.f, 0.f, 0.f);
-                if (MODE != RED_DISK_MINMAX) {
+            if (xa < xb) {
+                cnt += xb - xa;
+                int va, vb;
+                vector_span(f, xa, xb, &va, &vb);
+                // the columns outside the aligned middle: lane by lane
+                for (int x = xa + l; x < va; x += 32) add(__ldg(f + x), MODE != RED_DISK_MINMAX ? __ldg(g + x) : 0.f);
+                for (int x = vb + l; x < xb; x += 32) add(__ldg(f + x), MODE != RED_DISK_MINMAX ? __ldg(g + x) : 0.f);
+                const bool gvec = ((reinterpret_cast<uintptr_t>(g + va)) & 15) == 0;
+                const int nv = (vb - va) >> 2;
+                for (int v0 = l; v0 < nv; v0 += 32 * U) {
+                    float4 fv[U], gv[U];
 #pragma unroll
                     for (int u = 0; u < U; ++u)
-                        if (v0 + 32 * u < nv) {
-                            const float* gp = g + va + 4 * (v0 + 32 * u);
-                            if (gvec) gv[u] = __ldg(reinterpret_cast<const float4*>(gp));
-                            else gv[u] = make_float4(__ldg(gp), __ldg(gp + 1), __ldg(gp + 2), __ldg(gp + 3));
-                        }
-                }
+                        if (v0 + 32 * u < nv) fv[u] = __ldg(reinterpret_cast<const float4*>(f + va) + v0 + 32 * u);
 #pragma unroll
-                for (int u = 0; u < U; ++u)
-                    if (v0 + 32 * u < nv) {
-                        add(fv[u].x, gv[u].x);
-                        add(fv[u].y, gv[u].y);
-                        add(fv[u].z, gv[u].z);
-                        add(fv[u].w, gv[u].w);
+                    for (int u = 0; u < U; ++u) gv[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+                    if (MODE != RED_DISK_MINMAX) {
+#pragma unroll
+                        for (int u = 0; u < U; ++u)
+                            if (v0 + 32 * u < nv) {
+                                const float* gp = g + va + 4 * (v0 + 32 * u);
+                                if (gvec) gv[u] = __ldg(reinterpret_cast<const float4*>(gp));
+                                else gv[u] = make_float4(__ldg(gp), __ldg(gp + 1), __ldg(gp + 2), __ldg(gp + 3));
+                            }
                     }
+                    if (MODE == RED_DISK_MINMAX) {
+#pragma unroll
+                        for (int u = 0; u < U; ++u)
+                            if (v0 + 32 * u < nv) {
+                                mn = fminf(fminf(mn, fminf(fv[u].x, fv[u].y)), fminf(fv[u].z, fv[u].w));
+                                mx = fmaxf(fmaxf(mx, fmaxf(fv[u].x, fv[u].y)), fmaxf(fv[u].z, fv[u].w));
+                            }
+                    } else {
+                        float d2[2], f2[2];
+                        word(fv[0], gv[0], &d2[0], &f2[0]);
+                        if (v0 + 32 < nv) {
+                            word(fv[1], gv[1], &d2[1], &f2[1]);
+                            d2[0] += d2[1];
+                            f2[0] += f2[1];
+                        }
+                        s0 += d2[0];
+                        s1 += f2[0];
+                    }
+                }
             }
+            if (--left) {
+                yl += (long long)parts * RED_WARPS;
+                continue;
+            }
+            // the part's rows are done: its sums over the warp, both in one tree
+            if (MODE != RED_DISK_MINMAX) {
+                float v = (l & 16) ? s1 : s0;
+                v += __shfl_xor_sync(0xffffffffu, (l & 16) ? s0 : s1, 16);
+                for (int o = 8; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+                if ((l & 15) == 0) sh[l >> 4][part][w] = v;
+                s0 = s1 = 0.f;
+            }
+            left = per;
+            ++part;
+            first += (long long)blocks * RED_WARPS;
+            yl = first;
         }
     }
-    if (!waited) {                     // a warp without rows
-        griddep_wait();
-        griddep_launch();
-    }
-    __shared__ float sh[3][RED_WARPS];
-    __shared__ long long shc[RED_WARPS];
-    __shared__ int is_last;
-    s0 = warp_sum(s0);
-    s1 = warp_sum(s1);
+    // maximum, minimum and count go with the block's first part
     mx = warp_max(mx);
-    mn = warp_min(mn);
+    if (MODE == RED_DISK_MINMAX) mn = warp_min(mn);
     if (l == 0) {
-        sh[0][w] = s0;
-        sh[1][w] = MODE == RED_DISK_MINMAX ? mn : s1;
-        sh[2][w] = mx;
+        shm[0][w] = mx;
+        shm[1][w] = mn;
         shc[w] = cnt;
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
+    if (threadIdx.x < mine) {
+        const int v = threadIdx.x;
         double a = 0, c1 = MODE == RED_DISK_MINMAX ? (double)INFINITY : 0;
         float m2 = -INFINITY;
         long long n = 0;
         for (int j = 0; j < RED_WARPS; ++j) {
-            a += sh[0][j];
-            if (MODE == RED_DISK_MINMAX) c1 = fmin(c1, (double)sh[1][j]);
-            else c1 += sh[1][j];
-            m2 = fmaxf(m2, sh[2][j]);
-            n += shc[j];
+            if (MODE != RED_DISK_MINMAX) {
+                a += sh[0][v][j];
+                c1 += sh[1][v][j];
+            }
+            if (v == 0) {
+                if (MODE == RED_DISK_MINMAX) c1 = fmin(c1, (double)shm[1][j]);
+                m2 = fmaxf(m2, shm[0][j]);
+                n += shc[j];
+            }
         }
-        double* o = p.part + ((size_t)bl * gridDim.x + blockIdx.x) * 4;
+        double* o = p.part + ((size_t)bl * RED_MAX_PARTS + blockIdx.x + (size_t)v * blocks) * 4;
         *reinterpret_cast<double2*>(o) = make_double2(a, c1);
         *reinterpret_cast<double2*>(o + 2) = make_double2((double)m2, (double)n);
         __threadfence();
-        is_last = atomicAdd(p.done, 1) == (int)(gridDim.x * gridDim.y) - 1;
     }
     __syncthreads();
-    if (!is_last) return;
-    // out = (eps_1, eps, f_max, count), mm = (min, max): a warp per image,
-    // lanes over its records, then a shuffle tree
+    if (threadIdx.x == 0) is_last = atomicAdd(p.done + bl, 1) == blocks - 1;
+    __syncthreads();
+    if (!is_last || w) return;
+    // out = (eps_1, eps, f_max, count), mm = (min, max): lanes over the image's
+    // records, then a shuffle tree.  Every image has its own last block: one for
+    // all of a launch's images took 128 of them in turn (64 x 64 pixels each: 72 us a
+    // call, now 10).
     __threadfence();
-    for (int j = w; j < p.nb; j += RED_WARPS) {
-        double sd = 0, sf = 0, n = 0, dmx = -INFINITY, dmn = INFINITY;
-        const double2* rec = reinterpret_cast<const double2*>(p.part) + (size_t)j * gridDim.x * 2;
-        for (int e0 = l; e0 < (int)gridDim.x; e0 += 128) {      // four records in flight per lane
-            double2 ra[4], rb[4];
+    double sd = 0, sf = 0, n = 0, dmx = -INFINITY, dmn = INFINITY;
+    const double2* rec = reinterpret_cast<const double2*>(p.part) + (size_t)bl * RED_MAX_PARTS * 2;
+    for (int e0 = l; e0 < parts; e0 += 128) {       // four records in flight per lane
+        double2 ra[4], rb[4];
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const bool on = e0 + 32 * u < (int)gridDim.x;
-                ra[u] = on ? __ldcg(rec + 2 * (e0 + 32 * u))
-                           : make_double2(0, MODE == RED_DISK_MINMAX ? (double)INFINITY : 0);
-                rb[u] = on ? __ldcg(rec + 2 * (e0 + 32 * u) + 1) : make_double2(-(double)INFINITY, 0);
-            }
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                if (MODE == RED_DISK_MINMAX) {
-                    dmn = fmin(dmn, ra[u].y);
-                } else {
-                    sd += ra[u].x;
-                    sf += ra[u].y;
-                    n += rb[u].y;
-                }
-                dmx = fmax(dmx, rb[u].x);
-            }
+        for (int u = 0; u < 4; ++u) {
+            const bool on = e0 + 32 * u < parts;
+            ra[u] = on ? __ldcg(rec + 2 * (e0 + 32 * u))
+                       : make_double2(0, MODE == RED_DISK_MINMAX ? (double)INFINITY : 0);
+            rb[u] = on ? __ldcg(rec + 2 * (e0 + 32 * u) + 1) : make_double2(-(double)INFINITY, 0);
         }
-        for (int o = 16; o; o >>= 1) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
             if (MODE == RED_DISK_MINMAX) {
-                dmn = fmin(dmn, __shfl_xor_sync(0xffffffffu, dmn, o));
+                dmn = fmin(dmn, ra[u].y);
             } else {
-                sd += __shfl_xor_sync(0xffffffffu, sd, o);
-                sf += __shfl_xor_sync(0xffffffffu, sf, o);
-                n += __shfl_xor_sync(0xffffffffu, n, o);
+                sd += ra[u].x;
+                sf += ra[u].y;
+                n += rb[u].y;
             }
-            dmx = fmax(dmx, __shfl_xor_sync(0xffffffffu, dmx, o));
-        }
-        if (l) continue;
-        const size_t bj = (size_t)(p.b_off + j);
-        if (MODE == RED_DISK_MINMAX) {
-            p.mm[2 * bj] = (float)dmn;
-            p.mm[2 * bj + 1] = (float)dmx;
-        } else {
-            p.out[4 * bj + 0] = sd / sf;
-            p.out[4 * bj + 1] = sd / (dmx * dmx * n);
-            p.out[4 * bj + 2] = dmx;
-            p.out[4 * bj + 3] = n;
+            dmx = fmax(dmx, rb[u].x);
         }
     }
-    if (threadIdx.x == 0) *p.done = 0;
+    for (int o = 16; o; o >>= 1) {
+        if (MODE == RED_DISK_MINMAX) {
+            dmn = fmin(dmn, __shfl_xor_sync(0xffffffffu, dmn, o));
+        } else {
+            sd += __shfl_xor_sync(0xffffffffu, sd, o);
+            sf += __shfl_xor_sync(0xffffffffu, sf, o);
+            n += __shfl_xor_sync(0xffffffffu, n, o);
+        }
+        dmx = fmax(dmx, __shfl_xor_sync(0xffffffffu, dmx, o));
+    }
+    if (l) return;
+    p.done[bl] = 0;
+    const size_t bj = (size_t)b;
+    if (MODE == RED_DISK_MINMAX) {
+        p.mm[2 * bj] = (float)dmn;
+        p.mm[2 * bj + 1] = (float)dmx;
+    } else {
+        p.out[4 * bj + 0] = sd / sf;
+        p.out[4 * bj + 1] = sd / (dmx * dmx * n);
+        p.out[4 * bj + 2] = dmx;
+        p.out[4 * bj + 3] = n;
+    }
 }
 
 // out[b] = (eps_1, eps, f_max, count) from the nrec ring records (sd, sf,
@@ -865,14 +934,6 @@ k_reduce_records(const float4* __restrict__ part, int nrec, double count, double
     }
 }
 
-// Blocks per image of the row kernels: a row per warp where the device holds
-// that many at once (a second row for a few of the warps would double the
-// time), at least one block an image.
-static int row_blocks(zm_plan_t p, int rows, int nb) {
-    const int want = std::max(1, RED_PER_SM * num_sms(p->device) / nb);
-    return std::min(std::min(RED_MAX_BLOCKS, want), std::max(1, (rows + RED_WARPS - 1) / RED_WARPS));
-}
-
 template <int MODE>
 static int run_reduce(zm_plan_t p, const zm_image_t* ref, const zm_image_t* tst, const float* fhat,
                       const float* frec, int batch, double* out, float* mm, cudaStream_t st) {
@@ -883,12 +944,11 @@ static int run_reduce(zm_plan_t p, const zm_image_t* ref, const zm_image_t* tst,
     rp.out = out;
     rp.mm = mm;
     rp.done = p->work + 2;
-    int s = p->ws_red.grow(sizeof(double) * 4 * RED_MAX_BLOCKS * (size_t)std::min(batch, KD_MAX_IMG));
+    int s = p->ws_red.grow(sizeof(double) * 4 * RED_MAX_PARTS * (size_t)std::min(batch, KD_MAX_IMG));
     if (s != ZM_OK) return s;
     for (int b0 = 0; b0 < batch; b0 += KD_MAX_IMG) {
         const int nb = std::min(KD_MAX_IMG, batch - b0);
         rp.b_off = b0;
-        rp.nb = nb;
         int rows = MODE == RED_POLAR_ERRORS ? (rp.n_nodes + RED_SEG - 1) / RED_SEG : 1;
         if (MODE != RED_POLAR_ERRORS) {
             for (int j = 0; j < nb; ++j) {
@@ -901,8 +961,9 @@ static int run_reduce(zm_plan_t p, const zm_image_t* ref, const zm_image_t* tst,
                 }
             }
         }
-        const int blocks = row_blocks(p, rows, nb);
         rp.part = (double*)p->ws_red.ptr;         // each launch finishes its own images
+        rp.share = std::max(1, RED_PER_SM * num_sms(p->device) / nb);
+        const int blocks = part_blocks(row_parts(rows), rp.share);
         ZM_LAUNCH_PDL("k_reduce", k_reduce<MODE>, dim3(blocks, nb), dim3(RED_THREADS), 0, st, rp);
     }
     return ZM_OK;
@@ -924,6 +985,13 @@ struct NormParams {
     int b_off;
     CanvasDesc cv[KD_MAX_IMG];
 };
+
+// Blocks per image of k_minmax_apply: a row per warp where the device holds that
+// many at once (a second row for a few of the warps would double the time), at
+// least one block an image.
+static int apply_blocks(zm_plan_t p, int rows, int nb) {
+    return std::min(row_parts(rows), std::max(1, RED_PER_SM * num_sms(p->device) / nb));
+}
 
 // Rows as in k_reduce: a warp per row, only the disk's columns, 16-byte loads
 // and stores, the scale once per warp (three 3840 x 2160 bands: 62 us with a
@@ -981,7 +1049,7 @@ int launch_minmax_normalize(zm_plan_t p, const zm_canvas_t* cv, int batch, const
             np.cv[j] = resolve_canvas(cv[b0 + j]);
             hmax = std::max(hmax, np.cv[j].h);
         }
-        ZM_LAUNCH_PDL("k_minmax_apply", k_minmax_apply, dim3(row_blocks(p, hmax, nb), nb), dim3(RED_THREADS), 0, st, np);
+        ZM_LAUNCH_PDL("k_minmax_apply", k_minmax_apply, dim3(apply_blocks(p, hmax, nb), nb), dim3(RED_THREADS), 0, st, np);
     }
     return ZM_OK;
 }

@@ -192,8 +192,8 @@ struct zm_plan_s {
     zm::Workspace ws_scale;     // per-image min / max (normalisation)
     zm::Workspace ws_Fblk;      // ring spectra as bf16 hi / lo operand blocks (blocked projection)
     int* status = nullptr;      // device status word: ZM_ETIMEOUT after a timed-out wait
-    int* work = nullptr;        // device {next item, CTAs done} of the inverse ring FFT and {blocks done} of the
-                                // reductions, 0 between launches
+    int* work = nullptr;        // device {next item, CTAs done} of the inverse ring FFT and, for each image of a
+                                // launch, {blocks done} of the reductions; 0 between launches
     // launch choices
     int kb_rings = 8;           // rings per CTA in the resample + FFT kernel
     // set by the batch autotuner (0 = built-in heuristic)
@@ -311,7 +311,8 @@ inline GeoImage resolve(const zm_image_t& im) {
 
 int check_images(const zm_image_t* imgs, int batch);
 
-constexpr int RED_MAX_BLOCKS = 512;   // blocks (records) per image of the pixel and node reductions
+constexpr int RED_MAX_PARTS = 1024;   // parts (records) per image of the pixel and node reductions
+constexpr int KD_MAX_IMG = 128;       // images per launch of the pixel passes
 
 constexpr long long GATHER_PDL_SAMPLES = 1ll << 18;   // largest gather (samples) launched before its predecessor ends
 
