@@ -302,7 +302,8 @@ typedef struct zm_batch_s* zm_batch_t;
  * (resampling by TMA tiles or by the fused gather kernel, rings per CTA of the
  * ring FFT, radial split of the projection) are picked by timing candidates on
  * the given images, or read from the JSON cache named by the environment
- * variable ZM_TUNE_CACHE (which is then updated).  Synchronous; allocates.
+ * variable ZM_TUNE_CACHE (which is then updated).  A resampling path asked for
+ * with ZM_FUSED, ZM_RING_DFT or ZM_POLAR_DFT is taken without timing others.  Synchronous; allocates.
  *  plan_flags: one ZM_GRID_* | one ZM_PREC_*, for every group.
  */
 int zm_batch_create(zm_batch_t* batch, const zm_request_t* reqs, int count, unsigned plan_flags);

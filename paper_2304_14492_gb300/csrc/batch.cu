@@ -182,6 +182,10 @@ static int upload_copies(zm_batch_t b, const zm_request_t* reqs) {
 // the projection's CTAs-per-SM target for its radial split.  Results are kept
 // in a flat JSON object, one entry per line:
 //   "key": {"gather": g, "rings": r, "split": s, "us": t},
+// The key starts with the version of what an entry means (2: gather 0 is "staged
+// where images can be", which entries without a version left to the plan's own
+// rule; those are kept in the file and not read) and holds the transforms that the
+// environment asked of the plan.
 struct TuneChoice {
     int gather = 0, rings = 0, split = 0;
     double us = 0;
@@ -199,9 +203,20 @@ static std::string tune_key(zm_plan_t p, int batch, const GeoImage& g) {
     int bb = 1;
     while (bb < batch) bb <<= 1;
     char buf[256];
-    snprintf(buf, sizeof buf, "sm%d%d|nrho=%d|ntheta=%d|nmax=%d|batch=%d|prec=%d|grid=%d|img=%dx%d", major, minor,
-             p->n_rho, p->n_theta, p->n_max, bb, p->prec, p->grid, g.h, g.w);
+    snprintf(buf, sizeof buf, "v2|sm%d%d|nrho=%d|ntheta=%d|nmax=%d|batch=%d|prec=%d|grid=%d|img=%dx%d|fused=%d|dft=%d,%d",
+             major, minor, p->n_rho, p->n_theta, p->n_max, bb, p->prec, p->grid, g.h, g.w, p->fused_mode, p->dft_mode,
+             p->pdft_mode);
     return buf;
+}
+
+// A plan told to fuse or not to, or to use a tensor-core transform (ZM_FUSED,
+// ZM_RING_DFT, ZM_POLAR_DFT), does that: its resampling path is not a candidate.
+static bool path_told(zm_plan_t p) { return p->fused_mode != 0 || p->dft_mode > 0 || p->pdft_mode > 0; }
+
+static void apply_choice(zm_plan_t p, const TuneChoice& c) {
+    p->tune_gather = path_told(p) ? 0 : (c.gather ? 1 : 2);
+    p->tune_rings = c.rings;
+    p->tune_split = c.split;
 }
 
 static std::map<std::string, TuneChoice> read_tune_cache(const char* path) {
@@ -268,9 +283,7 @@ static int tune_group(zm_batch_t b, BatchGroup& g, const zm_request_t* reqs,
     const std::string key = tune_key(g.plan, (int)g.members.size(), geo);
     auto it = cache.find(key);
     if (it != cache.end()) {
-        g.plan->tune_gather = it->second.gather ? 1 : 2;
-        g.plan->tune_rings = it->second.rings;
-        g.plan->tune_split = it->second.split;
+        apply_choice(g.plan, it->second);
         return ZM_OK;
     }
     bool tma = true;
@@ -281,24 +294,21 @@ static int tune_group(zm_batch_t b, BatchGroup& g, const zm_request_t* reqs,
     // better than the staged ones, whatever each takes alone (256 requests: 158
     // us a replay, 186 staged); rings and split matter only to FP32 spectra and to
     // the split-K projection
-    const int first = g.plan->n_theta <= 256 ? 1 : 0;
+    const bool told = path_told(g.plan);
+    const int first = !told && g.plan->n_theta <= 256 ? 1 : 0;
     const bool blocked = blocked_projection(g.plan);
-    for (int gather = first; gather <= (tma ? 1 : first); ++gather)
+    for (int gather = first; gather <= (tma && !told ? 1 : first); ++gather)
         for (int rings : {2, 4, 8})
             for (int split : {4, 8}) {
                 if (blocked && (rings < 8 || split < 8)) continue;
                 if (split > 4 && g.plan->prec == PREC_FP32) continue;      // no radial split there
-                g.plan->tune_gather = gather ? 1 : 2;
-                g.plan->tune_rings = rings;
-                g.plan->tune_split = split;
+                apply_choice(g.plan, TuneChoice{gather, rings, split, 0});
                 double us = 0;
                 const int s = time_group(b, g, reqs, &us);
                 if (s != ZM_OK) return s;
                 if (us < best.us) best = TuneChoice{gather, rings, split, us};
             }
-    g.plan->tune_gather = best.gather ? 1 : 2;
-    g.plan->tune_rings = best.rings;
-    g.plan->tune_split = best.split;
+    apply_choice(g.plan, best);
     cache[key] = best;
     *changed = true;
     return ZM_OK;
