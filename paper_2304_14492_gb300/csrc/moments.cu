@@ -404,18 +404,14 @@ static int blk_slots(const KbParams& kp, size_t* smem) {
     cudaGetDevice(&dev);
     static std::mutex mu;
     static std::map<std::pair<int, size_t>, int> resident;     // (device, smem) -> CTAs on the device
-    static size_t configured[64] = {0};
+    static SharedMemoryLimit limit;
     std::lock_guard<std::mutex> lk(mu);
     auto it = resident.find({dev, *smem});
     if (it != resident.end()) return it->second;
-    if (*smem > 48 * 1024 && (dev >= 64 || *smem > configured[dev])) {
-        const cudaError_t e = cudaFuncSetAttribute(k_ring_blk<LOGN, IPI>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                   (int)*smem);
-        if (e != cudaSuccess) {
-            cuda_error(e, "cudaFuncSetAttribute(k_ring_blk)");
-            return 0;
-        }
-        if (dev < 64) configured[dev] = *smem;
+    const cudaError_t e = allow_smem(limit, k_ring_blk<LOGN, IPI>, dev, *smem);
+    if (e != cudaSuccess) {
+        cuda_error(e, "cudaFuncSetAttribute(k_ring_blk)");
+        return 0;
     }
     int per_sm = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_ring_blk<LOGN, IPI>, 256, *smem) != cudaSuccess ||
@@ -476,12 +472,8 @@ static int launch_kb_t(const KbParams& kp, int R, int nb, cudaStream_t st) {
                         (MODE == KB_RESAMPLE ? 0 : sizeof(float2) * ((size_t)FFT::TW_FLOAT2 + kp.n_max + 1));
     int dev = 0;
     cudaGetDevice(&dev);
-    static size_t configured[64] = {0};
-    if (smem > 48 * 1024 && (dev >= 64 || smem > configured[dev])) {
-        ZM_CUDA_TRY(cudaFuncSetAttribute(k_ring_spectra<LOGN, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem));
-        if (dev < 64) configured[dev] = smem;
-    }
+    static SharedMemoryLimit limit;
+    ZM_CUDA_TRY(allow_smem(limit, k_ring_spectra<LOGN, MODE>, dev, smem));
     static std::mutex mu;
     static std::map<std::pair<int, size_t>, int> resident;   // (R, smem) -> CTAs per SM
     int per_sm = 0;

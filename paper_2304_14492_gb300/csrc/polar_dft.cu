@@ -355,12 +355,9 @@ int launch_polar_dft(zm_plan_t p, const float* fhat, int b0, int nb, int batch, 
     if (s != ZM_OK) return s;
     const int ncols = dft_ncols(p->n_max);
     const size_t smem = pd_smem_bytes(2 * ncols);
-    static size_t configured[64] = {0};
+    static SharedMemoryLimit limit;
     const int dev = p->device;
-    if (dev < 0 || dev >= 64 || smem > configured[dev]) {
-        ZM_CUDA_TRY(cudaFuncSetAttribute(k_polar_dft, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        if (dev >= 0 && dev < 64) configured[dev] = smem;
-    }
+    ZM_CUDA_TRY(allow_smem(limit, k_polar_dft, dev, smem));
     PdParams kp;
     kp.fhat = fhat;
     kp.dft = p->dft32;

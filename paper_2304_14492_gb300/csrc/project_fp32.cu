@@ -168,12 +168,8 @@ static int launch_pf(const PfParams& pp, int dev, cudaStream_t st) {
     // shared memory then holds three CTAs of 32 columns per SM)
     const int W = (long long)(pp.n_max + 1) * tiles * ctiles <= 2 * num_sms(dev) ? 8 : 4;
     const size_t smem = sizeof(float) * W * 2 * (PF_ROWS + TN) * PF_PITCH;
-    static size_t configured[64] = {0};
-    if (smem > 48 * 1024 && (dev >= 64 || smem > configured[dev])) {
-        ZM_CUDA_TRY(
-            cudaFuncSetAttribute(k_project_fp32<TN, V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        if (dev < 64) configured[dev] = smem;
-    }
+    static SharedMemoryLimit limit;
+    ZM_CUDA_TRY(allow_smem(limit, k_project_fp32<TN, V>, dev, smem));
     ZM_LAUNCH_PDL("k_project_fp32", (k_project_fp32<TN, V>), dim3(ctiles, tiles, pp.n_max + 1), dim3(32 * W), smem, st,
                   pp);
     return ZM_OK;

@@ -334,12 +334,9 @@ int launch_projection_tc(zm_plan_t p, const float* F, int batch, float* out, uns
     const size_t cap = 227 * 1024;
     const size_t by_tmem = cap / (512 / ncols) + 1024;
     const size_t smem = std::max(need, std::min(cap, by_tmem));
-    static size_t configured[64] = {0};
+    static SharedMemoryLimit limit;
     int dev = p->device;
-    if (dev >= 64 || smem > configured[dev]) {
-        ZM_CUDA_TRY(cudaFuncSetAttribute(k_project_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        if (dev < 64) configured[dev] = smem;
-    }
+    ZM_CUDA_TRY(allow_smem(limit, k_project_tc, dev, smem));
     dim3 grid(p->n_max + 1, ctiles, S);
     ZM_LAUNCH_PDL("k_project_tc", k_project_tc, grid, dim3(TC_THREADS), smem, st, tp);
     const int tot = batch * p->P;
@@ -900,12 +897,9 @@ int launch_projection_blocked(zm_plan_t p, const uint8_t* Fblk, int batch, float
     while (ncols < (comb ? 2 * nt_max : nt_max)) ncols <<= 1;
     const size_t smem = std::max((size_t)bp.buf_off + (split ? tail2 : BLK_A_BYTES),
                                  (size_t)(228 * 1024 / 512 * ncols - 2048));
-    static size_t configured[64] = {0};
+    static SharedMemoryLimit limit;
     const int dev = p->device;
-    if (dev >= 64 || smem > configured[dev]) {
-        ZM_CUDA_TRY(cudaFuncSetAttribute(k_project_blk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        if (dev < 64) configured[dev] = smem;
-    }
+    ZM_CUDA_TRY(allow_smem(limit, k_project_blk, dev, smem));
     if (split) {
         cudaError_t e = launch_pdl_cluster(k_project_blk, dim3(p->n_max + 1, tiles, 2), dim3(TC_THREADS),
                                            dim3(1, 1, 2), smem, st, bp);

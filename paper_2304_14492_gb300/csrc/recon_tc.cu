@@ -287,12 +287,9 @@ int launch_radial_tc(zm_plan_t p, const float* moments, int batch, unsigned flag
     const size_t by_tmem = cap / (512 / ncols) + 1024;
     const size_t smem = std::max(need, std::min(cap, by_tmem));
     if (need > cap) return set_error(ZM_EUNSUPPORTED, "reconstruction blocks need %zu B of shared memory", need);
-    static size_t configured[64] = {0};
+    static SharedMemoryLimit limit;
     const int dev = p->device;
-    if (dev >= 64 || smem > configured[dev]) {
-        ZM_CUDA_TRY(cudaFuncSetAttribute(k_recon_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        if (dev < 64) configured[dev] = smem;
-    }
+    ZM_CUDA_TRY(allow_smem(limit, k_recon_tc, dev, smem));
     RtParams rp;
     rp.Rblk = p->Rblk;
     rp.rblk_off = p->rblk_off;

@@ -314,12 +314,8 @@ static int launch_ifft_t(const float* G, const float2* tw, int n_max, int n_rho,
     const size_t smem = sizeof(float2) * ((size_t)R * (n_max + 1) + FFT::TW_FLOAT2 + FFT::M + (size_t)R * FFT::TBUF);
     int dev = 0;
     cudaGetDevice(&dev);
-    static size_t configured[64] = {0};
-    if (smem > 48 * 1024 && (dev >= 64 || smem > configured[dev])) {
-        ZM_CUDA_TRY(cudaFuncSetAttribute(k_recon_ifft<LOGN, ERR>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem));
-        if (dev < 64) configured[dev] = smem;
-    }
+    static SharedMemoryLimit limit;
+    ZM_CUDA_TRY(allow_smem(limit, k_recon_ifft<LOGN, ERR>, dev, smem));
     const long long items = (long long)((n_rho + R - 1) / R) * batch;
     const int slots = sms * resident_blocks(k_recon_ifft<LOGN, ERR>, R * 32, smem);
     const int grid = (int)std::min<long long>(items, slots);
@@ -357,12 +353,8 @@ static int launch_radial_t(zm_plan_t p, const float* moments, int batch, unsigne
     const size_t smem = sizeof(float) * RR_WARPS * std::max(RR_RING, RB * 2 * RR_NODES) +
                         sizeof(float4) * RB * (size_t)(p->n_max / 2 + 1);
     const int dev = p->device;
-    static size_t configured[64] = {0};
-    if (smem > 48 * 1024 && (dev >= 64 || smem > configured[dev])) {
-        ZM_CUDA_TRY(
-            cudaFuncSetAttribute(k_recon_radial<RB, V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        if (dev < 64) configured[dev] = smem;
-    }
+    static SharedMemoryLimit limit;
+    ZM_CUDA_TRY(allow_smem(limit, k_recon_radial<RB, V>, dev, smem));
     const int nz = (batch + RB - 1) / RB;
     for (int z0 = 0; z0 < nz; z0 += 65535) {
         const int nzc = std::min(65535, nz - z0);

@@ -551,12 +551,9 @@ int launch_ring_dft(zm_plan_t p, const zm_image_t* imgs, int b0, int nb, int bat
     const int ncols = dft_ncols(p->n_max);
     const size_t smem = DfSmem::bytes(2 * ncols, dp->nstage);
     if (smem > 227 * 1024) return ZM_EUNSUPPORTED;
-    static size_t configured[64] = {0};
+    static SharedMemoryLimit limit;
     const int dev = p->device;
-    if (dev < 0 || dev >= 64 || smem > configured[dev]) {
-        ZM_CUDA_TRY(cudaFuncSetAttribute(k_ring_dft, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        if (dev >= 0 && dev < 64) configured[dev] = smem;
-    }
+    ZM_CUDA_TRY(allow_smem(limit, k_ring_dft, dev, smem));
     static thread_local DfParams kp;
     kp.stages = dp->stages;
     kp.rows = dp->rows;

@@ -561,11 +561,8 @@ template <int LOGN>
 static int launch_fused_t(zm_plan_t p, FuParams& fp_, int grid, cudaStream_t st) {
     const size_t smem = FuSmem<LOGN>::bytes(p->n_max);
     int dev = p->device;
-    static size_t configured[64] = {0};
-    if (smem > 48 * 1024 && (dev < 0 || dev >= 64 || smem > configured[dev])) {
-        ZM_CUDA_TRY(cudaFuncSetAttribute(k_ring_fused<LOGN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        if (dev >= 0 && dev < 64) configured[dev] = smem;
-    }
+    static SharedMemoryLimit limit;
+    ZM_CUDA_TRY(allow_smem(limit, k_ring_fused<LOGN>, dev, smem));
     ZM_LAUNCH_PDL("k_ring_fused", k_ring_fused<LOGN>, dim3(grid), dim3(FU_THREADS), smem, st, fp_);
     return ZM_OK;
 }

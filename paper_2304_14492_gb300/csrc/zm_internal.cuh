@@ -9,6 +9,7 @@
 #include <vector>
 
 #include "../../include/zm.h"
+#include "launch_limits.cuh"
 
 namespace zm {
 
@@ -92,6 +93,15 @@ inline cudaError_t launch_pdl_cluster(void (*kernel)(Params...), dim3 grid, dim3
         if (_e != cudaSuccess) return ::zm::cuda_error(_e, what);                     \
         ::zm::count_launch();                                                         \
     } while (0)
+
+// Lets `kernel` be launched with smem bytes of dynamic shared memory; `limit` is the
+// kernel's own (a static of the launcher).
+template <class K>
+inline cudaError_t allow_smem(SharedMemoryLimit& limit, K* kernel, int dev, size_t smem) {
+    return (cudaError_t)limit.raise(dev, smem, [&](size_t n) {
+        return (int)cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)n);
+    });
+}
 
 // Makes `dev` current for the lifetime of the guard and restores the caller's
 // device afterwards.
