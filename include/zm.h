@@ -115,7 +115,10 @@ int zm_plan(zm_plan_t* plan, int n_max, int n_rho, int n_theta, unsigned flags);
 int zm_plan_destroy(zm_plan_t plan);
 
 /* Grow the plan's workspace so that later calls with batch <= `batch`
- * allocate nothing (e.g. before CUDA graph capture).  Synchronous. */
+ * allocate nothing (e.g. before CUDA graph capture) but, on the first call with
+ * aligned images of a new geometry, that geometry's work list, which is built on a
+ * stream of its own and may be built while the caller's stream is captured.
+ * Synchronous. */
 int zm_plan_reserve(zm_plan_t plan, int batch);
 
 /* Synchronise the device, then report ZM_ETIMEOUT if any kernel of this plan

@@ -375,10 +375,12 @@ struct TileList {
 // within 2 px of the rectangle.
 static int build_tiles(zm_plan_t p, const GeoImage& g, TileList* tl) {
     const int N = p->n_theta, n_rho = p->n_rho;
+    SetupStream su;
+    ZM_CUDA_TRY(su.err);
     std::vector<double> rho(n_rho);
     {
         std::vector<float> r32(n_rho);
-        ZM_CUDA_TRY(cudaMemcpy(r32.data(), p->rho32, sizeof(float) * n_rho, cudaMemcpyDeviceToHost));
+        ZM_CUDA_TRY(su.to_host(r32.data(), p->rho32, sizeof(float) * n_rho));
         for (int i = 0; i < n_rho; ++i) rho[i] = (double)r32[i];
     }
     const double cx = g.cx, cy = g.cy, R = g.r;
@@ -450,7 +452,7 @@ static int build_tiles(zm_plan_t p, const GeoImage& g, TileList* tl) {
     tl->n = (int)h.size();
     if (!tl->n) return ZM_OK;
     ZM_CUDA_TRY(cudaMalloc(&tl->items, sizeof(TileItem) * h.size()));
-    ZM_CUDA_TRY(cudaMemcpy(tl->items, h.data(), sizeof(TileItem) * h.size(), cudaMemcpyHostToDevice));
+    ZM_CUDA_TRY(su.to_device(tl->items, h.data(), sizeof(TileItem) * h.size()));
     // plan: count the samples each tile owns, store them packed, then turn
     // them into records
     PlanParams pp;
@@ -465,10 +467,10 @@ static int build_tiles(zm_plan_t p, const GeoImage& g, TileList* tl) {
     pp.recs = nullptr;
     ZM_CUDA_TRY(cudaMalloc(&pp.counts, sizeof(int) * tl->n));
     pp.count_only = 1;
-    k_tile_plan<<<tl->n, TILE_THREADS>>>(pp);
+    k_tile_plan<<<tl->n, TILE_THREADS, 0, su.st>>>(pp);
     cudaError_t ce = cudaGetLastError();
     std::vector<int> cnt(tl->n);
-    if (ce == cudaSuccess) ce = cudaMemcpy(cnt.data(), pp.counts, sizeof(int) * tl->n, cudaMemcpyDeviceToHost);
+    if (ce == cudaSuccess) ce = su.to_host(cnt.data(), pp.counts, sizeof(int) * tl->n);
     cudaFree(pp.counts);
     if (ce != cudaSuccess) return cuda_error(ce, "k_tile_plan (count)");
     count_launch();
@@ -480,24 +482,23 @@ static int build_tiles(zm_plan_t p, const GeoImage& g, TileList* tl) {
     }
     if (total >= (1ll << 31)) return set_error(ZM_EINVAL, "too many polar samples for one geometry (%lld)", total);
     tl->n_samples = total;
-    ZM_CUDA_TRY(cudaMemcpy(tl->items, h.data(), sizeof(TileItem) * h.size(), cudaMemcpyHostToDevice));
+    ZM_CUDA_TRY(su.to_device(tl->items, h.data(), sizeof(TileItem) * h.size()));
     ZM_CUDA_TRY(cudaMalloc(&pp.samples, sizeof(uint32_t) * std::max<long long>(1, total)));
     ce = cudaMalloc(&tl->recs, sizeof(int4) * std::max<long long>(1, total));
     if (ce == cudaSuccess) {
         pp.recs = tl->recs;
         pp.count_only = 0;
-        k_tile_plan<<<tl->n, TILE_THREADS>>>(pp);
+        k_tile_plan<<<tl->n, TILE_THREADS, 0, su.st>>>(pp);
         ce = cudaGetLastError();
         if (ce == cudaSuccess) {
             count_launch();
-            k_tile_records<<<tl->n, TILE_THREADS>>>(pp);
+            k_tile_records<<<tl->n, TILE_THREADS, 0, su.st>>>(pp);
             ce = cudaGetLastError();
         }
-        if (ce == cudaSuccess) {
-            count_launch();
-            ce = cudaDeviceSynchronize();
-        }
+        if (ce == cudaSuccess) count_launch();
     }
+    const cudaError_t fe = su.finish();
+    if (ce == cudaSuccess) ce = fe;
     cudaFree(pp.samples);
     if (ce != cudaSuccess) return cuda_error(ce, "tile plan");
     return ZM_OK;

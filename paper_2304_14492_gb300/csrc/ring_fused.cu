@@ -401,10 +401,12 @@ struct Footprint {
 static int build_fused(zm_plan_t p, const GeoImage& g, FusedPlan* fp) {
     const int N = p->n_theta, n_rho = p->n_rho;
     const int nslot = N / FU_SLOT;
+    SetupStream su;
+    ZM_CUDA_TRY(su.err);
     std::vector<float> rho(n_rho);
     std::vector<float2> cs(N);
-    ZM_CUDA_TRY(cudaMemcpy(rho.data(), p->rho32, sizeof(float) * n_rho, cudaMemcpyDeviceToHost));
-    ZM_CUDA_TRY(cudaMemcpy(cs.data(), p->cs, sizeof(float2) * N, cudaMemcpyDeviceToHost));
+    ZM_CUDA_TRY(su.to_host(rho.data(), p->rho32, sizeof(float) * n_rho));
+    ZM_CUDA_TRY(su.to_host(cs.data(), p->cs, sizeof(float2) * N));
     fp->n_live = (n_rho + FU_R - 1) / FU_R;
     fp->n_all = std::max(fp->n_live, p->n_chunks * (64 / FU_R));
     std::vector<int2> band_st(fp->n_all, make_int2(0, 0));
@@ -497,13 +499,12 @@ static int build_fused(zm_plan_t p, const GeoImage& g, FusedPlan* fp) {
     ZM_CUDA_TRY(cudaMalloc(&fp->band_st, sizeof(int2) * band_st.size()));
     ZM_CUDA_TRY(cudaMalloc(&fp->stages, sizeof(FuStage) * std::max<size_t>(1, stages.size())));
     ZM_CUDA_TRY(cudaMalloc(&fp->rows, sizeof(int4) * std::max<size_t>(1, rows.size())));
-    ZM_CUDA_TRY(cudaMemcpy(fp->order, order.data(), sizeof(int) * order.size(), cudaMemcpyHostToDevice));
-    ZM_CUDA_TRY(cudaMemcpy(fp->order_live, order_live.data(), sizeof(int) * order_live.size(), cudaMemcpyHostToDevice));
-    ZM_CUDA_TRY(cudaMemcpy(fp->band_st, band_st.data(), sizeof(int2) * band_st.size(), cudaMemcpyHostToDevice));
-    if (!stages.empty())
-        ZM_CUDA_TRY(cudaMemcpy(fp->stages, stages.data(), sizeof(FuStage) * stages.size(), cudaMemcpyHostToDevice));
-    if (!rows.empty())
-        ZM_CUDA_TRY(cudaMemcpy(fp->rows, rows.data(), sizeof(int4) * rows.size(), cudaMemcpyHostToDevice));
+    ZM_CUDA_TRY(su.to_device(fp->order, order.data(), sizeof(int) * order.size()));
+    ZM_CUDA_TRY(su.to_device(fp->order_live, order_live.data(), sizeof(int) * order_live.size()));
+    ZM_CUDA_TRY(su.to_device(fp->band_st, band_st.data(), sizeof(int2) * band_st.size()));
+    if (!stages.empty()) ZM_CUDA_TRY(su.to_device(fp->stages, stages.data(), sizeof(FuStage) * stages.size()));
+    if (!rows.empty()) ZM_CUDA_TRY(su.to_device(fp->rows, rows.data(), sizeof(int4) * rows.size()));
+    ZM_CUDA_TRY(su.finish());
     fp->staged_floats = staged;
     fp->ok = true;
     return ZM_OK;

@@ -118,6 +118,33 @@ struct DeviceGuard {
     }
 };
 
+// A stream for building what a plan keeps per geometry, on first use of the
+// geometry, which may fall into the capture of the caller's stream (a call warmed up
+// with one image is captured with many, and takes another path): a stream of its own
+// that captures nothing and does not wait for the legacy stream, with this thread
+// allowed to allocate meanwhile.  finish() waits for it.
+struct SetupStream {
+    cudaStream_t st = nullptr;
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    cudaError_t err;
+    SetupStream() {
+        err = cudaThreadExchangeStreamCaptureMode(&mode);
+        if (err == cudaSuccess) err = cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking);
+    }
+    ~SetupStream() {
+        if (st) cudaStreamDestroy(st);
+        cudaThreadExchangeStreamCaptureMode(&mode);
+    }
+    cudaError_t to_host(void* dst, const void* src, size_t n) {
+        const cudaError_t e = cudaMemcpyAsync(dst, src, n, cudaMemcpyDeviceToHost, st);
+        return e == cudaSuccess ? finish() : e;
+    }
+    cudaError_t to_device(void* dst, const void* src, size_t n) {
+        return cudaMemcpyAsync(dst, src, n, cudaMemcpyHostToDevice, st);
+    }
+    cudaError_t finish() { return cudaStreamSynchronize(st); }
+};
+
 // ---------------------------------------------------------------- index set
 // Stored pairs (n, m): m >= 0, n - m even, ordered by n then m (Sec. 2).
 inline int num_moments(int n_max) {
