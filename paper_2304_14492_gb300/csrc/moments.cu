@@ -33,7 +33,8 @@ struct KbParams {
     GeoImage img[KB_MAX_IMG];
 };
 
-enum { KB_GATHER = 0, KB_POLAR = 1, KB_RESAMPLE = 2 };
+// KB_TILED: polar samples that the tile resampler has just written (1024 angles)
+enum { KB_GATHER = 0, KB_POLAR = 1, KB_RESAMPLE = 2, KB_TILED = 3 };
 
 // Bilinear value at pixel coordinates (X, Y); neighbours outside the image are 0.
 __device__ __forceinline__ float bilinear(const GeoImage& im, float X, float Y) {
@@ -94,11 +95,22 @@ __device__ __forceinline__ bool ring_inside(const GeoImage& im, float rad) {
 // Residency: four CTAs per SM up to 512 angles.  At 1024 the 64 registers that
 // leaves cost the gather its loads in flight and, with 32 rings at once, its hits
 // in L1: 8 images of 2161 x 2161 on 1024 x 1024 took 248 us, with two CTAs 67.
+// So do a caller's polar samples (16 images of 1024 x 1024 samples 42.1 us a call
+// with the projection, FP32; with four CTAs 44.6), but not what the tile resampler
+// leaves: there the wider CTAs, launched while it runs, take its place (FP32 spectra
+// of two 1024 x 1024 images on 1024 x 1024: 23.7 us a call, with four CTAs 17.5; from
+// eight such images on two are ahead again, 41.2 and 43.3).
+constexpr int kb_ctas(int logn, int mode) {
+    return logn >= 11 || (logn == 10 && mode != KB_RESAMPLE && mode != KB_TILED) ? 2 : 4;
+}
+constexpr long long TILED_SAMPLES = 3ll << 21;    // calls of more samples take KB_POLAR after the tiles
+
 template <int LOGN, int MODE>
-__global__ void __launch_bounds__(256, (LOGN >= 10 ? 2 : 4)) k_ring_spectra(const __grid_constant__ KbParams p) {
+__global__ void __launch_bounds__(256, kb_ctas(LOGN, MODE)) k_ring_spectra(const __grid_constant__ KbParams p) {
     using FFT = RingFFT<LOGN>;
     constexpr int N = FFT::N;
     constexpr int ROW = FFT::ROW_FLOATS;
+    constexpr bool POLAR = MODE == KB_POLAR || MODE == KB_TILED;
     extern __shared__ __align__(16) float smem[];
     const int R = blockDim.x >> 5;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -139,7 +151,7 @@ __global__ void __launch_bounds__(256, (LOGN >= 10 ? 2 : 4)) k_ring_spectra(cons
     };
     griddep_wait();                // the images or polar samples are written, the spectra are free
     griddep_launch();              // (the grid is resident at once)
-    if (MODE == KB_POLAR && (int)blockIdx.x < n_items) load_ring(blockIdx.x);
+    if (POLAR && (int)blockIdx.x < n_items) load_ring(blockIdx.x);
     bool ready = false;
     for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
         const int bl = item / n_rb;
@@ -210,7 +222,7 @@ __global__ void __launch_bounds__(256, (LOGN >= 10 ? 2 : 4)) k_ring_spectra(cons
                 for (int r = 0; r < FFT::Q; ++r) X[FFT::pad(FFT::fwd_index(r, lane))] = v[r];
             }
             __syncwarp();
-            if (MODE == KB_POLAR && item + (int)gridDim.x < n_items) load_ring(item + gridDim.x);
+            if (POLAR && item + (int)gridDim.x < n_items) load_ring(item + gridDim.x);
             for (int m = lane; m <= n_max; m += 32) {
                 const float2 A = X[FFT::pad(m)];
                 const float2 B = cconj(X[FFT::pad((FFT::M - m) & (FFT::M - 1))]);
@@ -495,10 +507,12 @@ static int launch_kb_t(const KbParams& kp, int R, int nb, cudaStream_t st) {
     const long long items = (long long)(kp.Fblk ? kp.n_chunks * (64 / R) : (kp.n_rho + R - 1) / R) * nb;
     const int grid = (int)std::min<long long>(items, (long long)per_sm * num_sms(dev));
     // A gather of more than GATHER_PDL_SAMPLES is not launched early: it lives on
-    // L1, and CTAs that come in while the previous call's projection holds most
-    // of the SM's shared memory keep that split for their lifetime (16 images of
-    // 512 x 512 on a 256 x 256 grid, back to back: 27 us a call with the early
-    // launch, 18 without; 40 images of 1024 x 1024 on 512 x 256, FP32: 164 and 62).
+    // L1, and CTAs that come in while the previous call's projection holds the SM's
+    // shared memory keep that split for their lifetime (zm_moments captured, with the
+    // early launch / without, us: 40 images of 1024 x 1024 on 512 x 256, bf16x3 149 / 54,
+    // fp16x3 151 / 69; 40 of 512 x 512 on 256 x 256, bf16x3 45 / 29; 1024 x 1024 on 512 x
+    // 1024, two images 26 / 17; half a million samples 0 to 13 % the same way, though
+    // uncaptured calls of that size gain 10 %).
     if (MODE == KB_GATHER && (long long)nb * kp.n_rho * FFT::N > GATHER_PDL_SAMPLES) {
         k_ring_spectra<LOGN, MODE><<<grid, R * 32, smem, st>>>(kp);
         ZM_LAUNCH_CHECK("k_ring_spectra");
@@ -525,14 +539,16 @@ static int launch_kb_mode(int logn, const KbParams& kp, int R, int nb, cudaStrea
 }
 
 // ============================================================== driver
-static int pick_rings(zm_plan_t p, int batch) {
+static int pick_rings(zm_plan_t p, int batch, bool tiled) {
     if (p->tune_rings == 2 || p->tune_rings == 4 || p->tune_rings == 8) return p->tune_rings;
     int R = 8;
     const int want = 2 * num_sms(p->device);
     // two rings to a CTA spread small calls over the SMs; rings of 512 angles and
     // more keep four (their twiddle tables are loaded by every CTA: one 2160 x
-    // 2160 image on 1024 x 1024, FP32, 20.8 us against 23.7 with two)
-    const int least = p->n_theta >= 512 ? 4 : 2;
+    // 2160 image on 1024 x 1024, FP32, 20.8 us against 23.7 with two), but after the
+    // tiles only where the rings are few (one 2160 x 2160 image on 256 x 2048 10.8
+    // us against 11.7; one 1024 x 1024 image on 512 x 2048 18.2 against 14.0 with two)
+    const int least = p->n_theta >= 512 && !(tiled && (long long)p->n_rho * batch > want) ? 4 : 2;
     while (R > least && ((p->n_rho + R - 1) / R) * batch < want) R >>= 1;
     return R;
 }
@@ -542,12 +558,12 @@ static int pick_rings(zm_plan_t p, int batch) {
 static int launch_gather(zm_plan_t p, const zm_image_t* imgs, int b0, int nb, int batch, float* F, float* fhat_out,
                          bool resample_only, uint8_t* Fblk, cudaStream_t st) {
     // operand blocks take whole rows of 8 rings; calls of few blocks are spread
-    // over twice the CTAs instead (us a call with 8 / 4 rings: one 256 x 256 image
+    // over twice the CTAs instead (us a call, not captured, with 8 / 4 rings: one 256 x 256 image
     // on 128 x 256 8.3 / 7.5, on 64 x 1024 11.7 / 9.3; one 1024 x 1024 on 512 x
     // 1024 19.2 / 16.1; beyond, the half rows cost more: four 256 x 256 images on
     // 128 x 128 7.1 / 7.4)
     const long long blocks = 8ll * p->n_chunks * batch;
-    const int R = Fblk ? (blocks <= (p->n_theta >= 1024 ? 64 : 32) ? 4 : 8) : pick_rings(p, batch);
+    const int R = Fblk ? (blocks <= (p->n_theta >= 1024 ? 64 : 32) ? 4 : 8) : pick_rings(p, batch, false);
     static thread_local KbParams kp;
     kp.Fblk = resample_only ? nullptr : Fblk;
     kp.fblk_half = fblk_half_bytes(p->n_max, p->n_chunks, 2 * batch);
@@ -575,11 +591,12 @@ static int launch_gather(zm_plan_t p, const zm_image_t* imgs, int b0, int nb, in
 
 // Angular transform of given polar samples fhat[b][i][k] -> F (or the
 // operand blocks Fblk) for images [b0, b0 + nb) of a batch of `batch`: the
-// tensor-core DFT where the plan allows it, else the ring FFT.
+// tensor-core DFT where the plan allows it, else the ring FFT.  tiled: the tile
+// resampler has just written them; scratch: into the plan's workspace.
 static int launch_polar_fft(zm_plan_t p, const float* fhat, int b0, int nb, int batch, float* F, uint8_t* Fblk,
-                            cudaStream_t st, bool scratch = false) {
+                            cudaStream_t st, bool tiled = false, bool scratch = false) {
     if (Fblk && polar_dft_eligible(p, fhat)) return launch_polar_dft(p, fhat, b0, nb, batch, Fblk, st);
-    const int R = Fblk ? 8 : pick_rings(p, batch);
+    const int R = Fblk ? 8 : pick_rings(p, batch, tiled);
     static thread_local KbParams kp;
     kp.Fblk = Fblk;
     kp.fblk_half = fblk_half_bytes(p->n_max, p->n_chunks, 2 * batch);
@@ -597,7 +614,10 @@ static int launch_polar_fft(zm_plan_t p, const float* fhat, int b0, int nb, int 
     for (int c0 = b0; c0 < b0 + nb; c0 += 65535) {
         const int nc = std::min(65535, b0 + nb - c0);
         kp.b_off = c0;
-        const int s = Fblk ? launch_blk(p->log_theta, kp, nc, st) : launch_kb_mode<KB_POLAR>(p->log_theta, kp, R, nc, st);
+        const bool narrow = tiled && p->log_theta == 10 && (long long)nc * p->n_rho * p->n_theta <= TILED_SAMPLES;
+        const int s = Fblk     ? launch_blk(p->log_theta, kp, nc, st)
+                      : narrow ? launch_kb_t<10, KB_TILED>(kp, R, nc, st)
+                               : launch_kb_mode<KB_POLAR>(p->log_theta, kp, R, nc, st);
         if (s != ZM_OK) return s;
     }
     return ZM_OK;
@@ -606,30 +626,38 @@ static int launch_polar_fft(zm_plan_t p, const float* fhat, int b0, int nb, int 
 // Where the gather kernel is the fastest of the three by default.  Its rings of
 // up to 256 angles leave a lane eight samples, whose loads are all in flight;
 // images come from L1 and L2, and no plan of tiles or stages stands before the
-// first pixel.  (At 256 angles and about a million samples in small grids the
-// staged kernel is ahead by 5 to 10 %; against the tiles of larger grids the
-// gather leads: 2160 x 2160 on 1080 x 256, 4 images 21.4 / 27.6.)  Measured per
-// call, back to back (gather / fused or tiles, us, bf16x3): 64 x 64 on 32 x 64, 1
-// image 5.5 / 6.6; 512 x 512 on 256 x 256, 4 images 9.8 / 16.0, 16 images 17.6 /
-// 16.5, 40 images 30.6 / 33.1; 1024 x 1024 on 512 x 256, 40 images 56.4 / 66.9;
-// 2160 x 2160 on 1080 x 256, 1 image 14.4 / 20.0, 16 images 59.6 / 63.5.  At 512 angles (16 samples a lane) it holds up to
-// about 1.5 million samples a call: 512 x 512 on 256 x 512, 4 images 12.7 / 20.2,
-// 8 images 16.0 / 20.5, 16 images 24.1 / 21.1 (grids of more than 2^17 samples
-// keep the tiles, whose lead at 8 images is as large).  At 1024 angles, with
-// operand blocks as output, up to the same number: 2160 x 2160 on 1024 x 1024,
-// 1 image 19.2 / 23.7, 4 images 42.7 / 34.8; 1024 x 1024 on 512 x 1024, 1 image
-// 26.8 / 30.9, 16 images 69 / 57.  With FP32 rows, whose ring FFT after the tiles
-// is cheaper, up to a third of it: 1024 x 1024 on 512 x 1024, 1 image 17.5 / 20.2;
-// 2160 x 2160 on 1024 x 1024, 1 image 20.8 / 18.6.  A plan told to fuse or not to
-// (ZM_FUSED), or to use a tensor-core transform, does that.
-static bool gather_by_default(zm_plan_t p, int batch) {
+// first pixel.  Measured per zm_moments call, captured and back to back (gather /
+// staged up to 2^17 samples an image, tiles above; us, bf16x3 unless said, sizes as
+// image side on N_rho x N_theta):
+//  256 angles: 256 on 128 x 256, 16 images 11.6 / 13.8; 700 on 350 x 256, 6 images
+//   12.8 / 17.4, 16 images 20.7 / 21.9; 1024 on 512 x 256, 6 images 15.7 / 19.5, 12
+//   images 22.5 / 25.1; 2160 on 1080 x 256, 4 images 21.9 / 27.6.  Only on grids of
+//   2^16 samples and about a million samples a call is the staged kernel ahead: 512
+//   on 256 x 256, 12 images 14.8 / 16.1, 16 images 17.1 / 16.2 (order 100: 19.5 /
+//   17.7), 40 images 29.1 / 33.1.
+//  512 angles (16 samples a lane), grids of up to 2^17 samples, up to 1.5 million a
+//   call: 512 on 256 x 512, 4 images 12.9 / 16.5, 8 images 17.3 / 16.9, 16 images
+//   25.5 / 21.7; FP32 16.3 / 19.3 and 23.6 / 21.4 with 8 and 16.
+//  1024 angles.  Grids of up to 2^17 samples would be staged, which is far slower
+//   there: up to 1.5 million a call (512 on 128 x 1024, 12 images 22.6 / 25.3, FP32
+//   20.5 / 25.7).  Larger grids have the tiles, and the form the spectra are wanted in
+//   decides.  Operand blocks: up to 1.25 million (512 on 256 x 1024, 4 images 21.7 /
+//   23.2, 6 images 28.6 / 27.8; 1024 on 512 x 1024, 2 images 17.1 / 22.7, 3 images 23.5
+//   / 22.8; 2160 on 1024 x 1024, 1 image 19.7 / 19.8).  FP32 rows, whose ring FFT
+//   after the tiles is cheaper: below a million (512 on 256 x 1024, 3 images 15.9 / 20.4;
+//   1024 on 512 x 1024, 1 image 12.9 / 15.1, 3 images 20.7 / 19.2; 2160 on 1024 x 1024,
+//   1 image 21.3 / 18.9).
+// A plan told to fuse or not to (ZM_FUSED), or to use a tensor-core transform, does
+// that.
+static bool gather_by_default(zm_plan_t p, int batch, bool operand_blocks) {
     if (p->fused_mode != 0 || p->dft_mode > 0 || p->pdft_mode > 0) return false;
-    const long long samples = (long long)p->n_rho * p->n_theta;
+    const long long samples = (long long)p->n_rho * p->n_theta, call = samples * batch;
     if (p->n_theta < 256) return true;
-    if (p->n_theta == 256)
-        return samples > FUSED_AUTO_SAMPLES || samples * batch <= 1ll << 19 || samples * batch > 3ll << 19;
-    if (p->n_theta == 512) return samples <= FUSED_AUTO_SAMPLES && samples * batch <= 3ll << 19;
-    return p->n_theta == 1024 && samples * batch <= (blocked_projection(p) ? 3ll << 19 : 1ll << 19);
+    if (p->n_theta == 256) return samples > 1 << 16 || call <= 7ll << 17 || call > 3ll << 19;
+    if (p->n_theta == 512) return samples <= FUSED_AUTO_SAMPLES && call <= 3ll << 19;
+    if (p->n_theta > 1024) return false;
+    if (samples <= FUSED_AUTO_SAMPLES) return call <= 3ll << 19;
+    return operand_blocks ? call <= 5ll << 18 : call < 1ll << 20;
 }
 
 // Ring spectra of a batch.  Polar input: FFT only.  Images: runs of one
@@ -646,7 +674,7 @@ int launch_spectra(zm_plan_t p, const zm_image_t* imgs, const float* fhat_in, in
     if (fhat_in) return launch_polar_fft(p, fhat_in, 0, batch, batch, F, Fblk, st);
     const bool fuse = p->fused_mode > 0 ||
                       (p->fused_mode == 0 && (long long)p->n_rho * p->n_theta <= FUSED_AUTO_SAMPLES);
-    const bool gather = p->tune_gather == 1 || (p->tune_gather == 0 && !resample_only && gather_by_default(p, batch));
+    const bool gather = p->tune_gather == 1 || (p->tune_gather == 0 && !resample_only && gather_by_default(p, batch, Fblk != nullptr));
     const bool dft = Fblk && !fhat_out && !resample_only && !gather && p->dft_mode > 0;
     auto use_dft = [&](int b) { return dft && dft_eligible(p, imgs[b]); };
     auto use_fused = [&](int b) { return fuse && !resample_only && !gather && fused_eligible(p, imgs[b]); };
@@ -689,7 +717,7 @@ int launch_spectra(zm_plan_t p, const zm_image_t* imgs, const float* fhat_in, in
             const bool scratch = fh != fhat_out && !resample_only;
             const bool keep = scratch && !(Fblk && polar_dft_eligible(p, fh));
             s = launch_resample_tiles(p, imgs, b, e - b, fh, st, keep);
-            if (s == ZM_OK && !resample_only) s = launch_polar_fft(p, fh, b, e - b, batch, F, Fblk, st, scratch);
+            if (s == ZM_OK && !resample_only) s = launch_polar_fft(p, fh, b, e - b, batch, F, Fblk, st, true, scratch);
         } else {
             while (e < batch && !use_tma(e)) ++e;
             s = launch_gather(p, imgs, b, e - b, batch, F, fhat_out, resample_only, Fblk, st);
