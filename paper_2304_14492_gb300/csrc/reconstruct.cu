@@ -20,7 +20,7 @@ constexpr float kTwoPi = 6.28318530717958647692f;
 // half sum over the stored m >= 0.
 //
 // Bound by reading the table once per RB images.  One CTA = 128 nodes, one m
-// and RB images (the fewest of 1, 2, 4, 8 that hold the batch); its eight warps
+// and RB images (the fewest of 1, 2, 4 that hold the batch); its eight warps
 // take every eighth order, so the longest chain is K_m / 8 steps and the few
 // heavy m do not outlast the rest, and their sums meet in shared memory in a
 // fixed order.  Each warp streams its own orders' rows through a ring of three
@@ -35,7 +35,7 @@ constexpr int RR_RING = RR_STAGES * RR_U * RR_NODES;      // floats of a warp's 
 
 // V: floats per copy (4, or 1 where rows are not 16-byte aligned).
 template <int RB, int V>
-__global__ void __launch_bounds__(32 * RR_WARPS, RB <= 4 ? 3 : 2)
+__global__ void __launch_bounds__(32 * RR_WARPS, 3)
 k_recon_radial(const float* __restrict__ R32m, const float2* __restrict__ Z, const int* __restrict__ mrow,
                int n_max, int n_rho, int P, int batch, int neumann, float* __restrict__ G) {
     extern __shared__ __align__(16) float rr_sm[];        // the rings, then the moments [RB][Km] (twice each)
@@ -129,6 +129,139 @@ k_recon_radial(const float* __restrict__ R32m, const float2* __restrict__ Z, con
         float v = 0.f;
         for (int w = 0; w < parts; ++w) v += rr_sm[w * OUT + e];
         G[g_index(b0 + (bc >> 1), i, m, bc & 1, nrb, n_max + 1)] = cm * v;
+    }
+}
+
+// The same sums for more than four images.  Splitting K_m over warps costs a pass
+// over all sums per eight images, which outweighs the sums themselves once the
+// images fill the device, so here a warp keeps all orders of 64 nodes and 8 images:
+// a lane has 8 nodes of one ring block (its share of G is one run of 64 bytes per
+// image, written a 32-byte sector at a time) and 2 images as (re, im) pairs, 16 packed
+// multiply-adds an order for three 16-byte shared-memory loads.  The CTA's warps are
+// IG groups of images by NG of nodes; rows come in chunks of eight orders through
+// three stages (cp.async), the moments of the next chunk are loaded while one is
+// multiplied.  A chunk's sums are taken apart and then added, so that no sum is a
+// longer chain than in k_recon_radial (8 + K_m / 8 additions).  Bound by shared-memory
+// bandwidth and FP32 issue.  zm_reconstruct, us a call, with the sums split over
+// warps for eight images / like this: n_max 60 on 256 nodes, 64 images 24.3 / 15.6; 127
+// on 512, 16 images 30.0 / 23.6, 128 images 204 / 126; 300 on 512, 8 images 38.5 / 32.6,
+// 128 images 568 / 340; 1000 on 256, 16 images 381 / 175 (a thread per node before
+// either: 16.9, 23.9, 131, 42.8, 390, 359).
+constexpr int RW_KC = 8, RW_STAGES = 3;
+
+template <int IG, int NG, int V>
+__global__ void __launch_bounds__(32 * IG * NG, 16 / (IG * NG))
+k_recon_radial_wide(const float* __restrict__ R32m, const float2* __restrict__ Z, const int* __restrict__ mrow,
+                    int n_max, int n_rho, int P, int batch, int neumann, float* __restrict__ G) {
+    constexpr int NODES = 64 * NG, IMGS = 8 * IG, THREADS = 32 * IG * NG;
+    __shared__ __align__(16) float rows[RW_STAGES][RW_KC][NODES];
+    __shared__ __align__(16) float2 zs[2][RW_KC][IMGS];
+    const int i0 = blockIdx.x * NODES, m = blockIdx.y, b0 = blockIdx.z * IMGS;
+    const int Km = (n_max - m) / 2 + 1, chunks = (Km + RW_KC - 1) / RW_KC;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int ig = warp % IG, nh = warp / IG;         // the warp's images and nodes
+    const int ng = lane & 7, cg = lane >> 3;          // the lane's ring block and pair of images
+    const float* Rm = R32m + (size_t)mrow[m] * n_rho + i0;
+    const uint32_t rows_a = static_cast<uint32_t>(__cvta_generic_to_shared(&rows[0][0][0]));
+    // 16-byte words of a row: within 64 nodes the even ones first, then the odd
+    // ones, so that the eight lanes of a phase read 128 consecutive bytes
+    auto place = [](int q) { return (q & ~15) + ((q & 1) << 3) + ((q & 15) >> 1); };
+    // the first order of the c-th chunk taken: the high orders first, whose moments
+    // are the smaller ones wherever they fall off
+    auto order0 = [&](int c) { return (chunks - 1 - c) * RW_KC; };
+    auto issue = [&](int c) {
+        if (c < chunks) {
+            const int j0 = order0(c), live = min(RW_KC, Km - j0), st = c % RW_STAGES;
+            for (int e = threadIdx.x; e < RW_KC * NODES / V; e += THREADS) {
+                const int k = e / (NODES / V), x = (e % (NODES / V)) * V;
+                if (k >= live) break;
+                const int on = i0 + x < n_rho;                        // else zero-filled
+                const float* src = on ? Rm + (size_t)(j0 + k) * n_rho + x : Rm;
+                const uint32_t dst = rows_a + 4u * ((st * RW_KC + k) * NODES + 4 * place(x >> 2) + (x & 3));
+                if (V == 4)
+                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(on ? 16 : 0)
+                                 : "memory");
+                else
+                    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(on ? 4 : 0)
+                                 : "memory");
+            }
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    // one moment per thread and chunk: order t / IMGS of the chunk, image t mod IMGS
+    const int zk = threadIdx.x / IMGS, zb = threadIdx.x % IMGS;
+    const float2* Zb = Z + (size_t)min(b0 + zb, batch - 1) * P;
+    auto moment = [&](int c) {
+        const int j = order0(c) + zk;
+        return c < chunks && zk < RW_KC && j < Km && b0 + zb < batch ? __ldg(Zb + moment_index(m + 2 * j, m)) : make_float2(0.f, 0.f);
+    };
+    issue(0);                          // the table is the plan's
+    issue(1);
+    griddep_wait();                    // the moments are written, G is free
+    griddep_launch();
+    float2 zn = moment(0);
+    if (zk < RW_KC) zs[0][zk][zb] = zn;
+    zn = moment(1);
+    const bool busy = b0 + ig * 8 < batch && i0 + nh * 64 < n_rho;
+    f32x2 tot[8][2];
+#pragma unroll
+    for (int r = 0; r < 8; ++r) tot[r][0] = tot[r][1] = 0;
+    for (int c = 0; c < chunks; ++c) {
+        asm volatile("cp.async.wait_group 1;" ::: "memory");
+        __syncthreads();               // chunk c is here; chunk c - 1 is read
+        issue(c + 2);
+        if (zk < RW_KC) zs[(c + 1) & 1][zk][zb] = zn;
+        zn = moment(c + 2);
+        if (!busy) continue;
+        const int live = min(RW_KC, Km - order0(c));
+        const float* rk = &rows[c % RW_STAGES][0][nh * 64 + 4 * ng];
+        const float2* zk_ = &zs[c & 1][0][ig * 8 + cg * 2];
+        f32x2 acc[8][2];
+#pragma unroll
+        for (int r = 0; r < 8; ++r) acc[r][0] = acc[r][1] = 0;
+#pragma unroll
+        for (int k = 0; k < RW_KC; ++k) {
+            if (k >= live) break;
+            const float4 a = *reinterpret_cast<const float4*>(rk + k * NODES);
+            const float4 b = *reinterpret_cast<const float4*>(rk + k * NODES + 32);
+            const ulonglong2 z = *reinterpret_cast<const ulonglong2*>(zk_ + k * IMGS);
+            const float r8[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+#pragma unroll
+            for (int r = 0; r < 8; ++r) {
+                const f32x2 rr = pack2(r8[r], r8[r]);
+                acc[r][0] = fma2(rr, z.x, acc[r][0]);
+                acc[r][1] = fma2(rr, z.y, acc[r][1]);
+            }
+        }
+#pragma unroll
+        for (int r = 0; r < 8; ++r) {
+            tot[r][0] = add2(tot[r][0], acc[r][0]);
+            tot[r][1] = add2(tot[r][1], acc[r][1]);
+        }
+    }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    const int i = i0 + nh * 64 + ng * 8;
+    if (!busy || i >= n_rho) return;
+    const float cm = (neumann && m > 0) ? 2.f : 1.f;
+    const int nrb = (n_rho + 7) / 8;
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+        const int b = b0 + ig * 8 + cg * 2 + e;
+        if (b >= batch) break;
+        float re[8], im[8];
+#pragma unroll
+        for (int r = 0; r < 8; ++r) {
+            const float2 v = unpack2(tot[r][e]);
+            re[r] = cm * v.x;
+            im[r] = cm * v.y;
+        }
+        // all 8 rings of the block (those past n_rho are zero and not read), a whole
+        // 32-byte sector at a time
+        float* g = G + g_index(b, i, m, 0, nrb, n_max + 1);
+        asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(g), "f"(re[0]), "f"(re[1]),
+                     "f"(re[2]), "f"(re[3]), "f"(re[4]), "f"(re[5]), "f"(re[6]), "f"(re[7]) : "memory");
+        asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(g + 8), "f"(im[0]), "f"(im[1]),
+                     "f"(im[2]), "f"(im[3]), "f"(im[4]), "f"(im[5]), "f"(im[6]), "f"(im[7]) : "memory");
     }
 }
 
@@ -348,6 +481,23 @@ static int launch_ifft(zm_plan_t p, const float* G, int batch, float* out, const
     }
 }
 
+template <int IG, int NG, int V>
+static int launch_radial_wide_t(zm_plan_t p, const float* moments, int batch, unsigned flags, float* G,
+                                cudaStream_t st) {
+    constexpr int NODES = 64 * NG, IMGS = 8 * IG;
+    const int nz = (batch + IMGS - 1) / IMGS;
+    for (int z0 = 0; z0 < nz; z0 += 65535) {
+        const int nzc = std::min(65535, nz - z0);
+        const int b0 = z0 * IMGS;
+        const int nbc = std::min(batch - b0, nzc * IMGS);
+        ZM_LAUNCH_PDL("k_recon_radial_wide", (k_recon_radial_wide<IG, NG, V>),
+                      dim3((p->n_rho + NODES - 1) / NODES, p->n_max + 1, nzc), dim3(32 * IG * NG), 0, st, (const float*)p->R32m,
+                      (const float2*)moments + (size_t)b0 * p->P, (const int*)p->mrow, p->n_max, p->n_rho, p->P, nbc,
+                      (flags & ZM_NEUMANN) ? 1 : 0, G + g_floats(b0, p->n_rho, p->n_max));
+    }
+    return ZM_OK;
+}
+
 template <int RB, int V>
 static int launch_radial_t(zm_plan_t p, const float* moments, int batch, unsigned flags, float* G, cudaStream_t st) {
     const size_t smem = sizeof(float) * RR_WARPS * std::max(RR_RING, RB * 2 * RR_NODES) +
@@ -378,10 +528,13 @@ static int launch_radial(zm_plan_t p, const float* moments, int batch, unsigned 
         return launch_radial_tc(p, moments, batch, flags, G, st);
     }
     const bool vec = (p->n_rho & 3) == 0;
+    // more than four images: all orders in a warp, 256 nodes to a CTA, or 128 where
+    // rows are copied float by float (its copies are four times as many)
     const int st_ = batch == 1   ? (vec ? launch_radial_t<1, 4> : launch_radial_t<1, 1>)(p, moments, batch, flags, G, st)
                     : batch == 2 ? (vec ? launch_radial_t<2, 4> : launch_radial_t<2, 1>)(p, moments, batch, flags, G, st)
                     : batch <= 4 ? (vec ? launch_radial_t<4, 4> : launch_radial_t<4, 1>)(p, moments, batch, flags, G, st)
-                                 : (vec ? launch_radial_t<8, 4> : launch_radial_t<8, 1>)(p, moments, batch, flags, G, st);
+                    : vec        ? launch_radial_wide_t<2, 4, 4>(p, moments, batch, flags, G, st)
+                                 : launch_radial_wide_t<2, 2, 1>(p, moments, batch, flags, G, st);
     if (st_ != ZM_OK) return st_;
     *G_out = G;
     return ZM_OK;
