@@ -20,7 +20,7 @@ constexpr float kTwoPi = 6.28318530717958647692f;
 // half sum over the stored m >= 0.
 //
 // Bound by reading the table once per RB images.  One CTA = 128 nodes, one m
-// and RB images (the fewest of 1, 2, 4 that hold the batch); its eight warps
+// and RB images (the fewest of 1, 2, 4 that hold the batch, or four); its eight warps
 // take every eighth order, so the longest chain is K_m / 8 steps and the few
 // heavy m do not outlast the rest, and their sums meet in shared memory in a
 // fixed order.  Each warp streams its own orders' rows through a ring of three
@@ -132,7 +132,7 @@ k_recon_radial(const float* __restrict__ R32m, const float2* __restrict__ Z, con
     }
 }
 
-// The same sums for more than four images.  Splitting K_m over warps costs a pass
+// The same sums for larger batches (launch_radial).  Splitting K_m over warps costs a pass
 // over all sums per eight images, which outweighs the sums themselves once the
 // images fill the device, so here a warp keeps all orders of 64 nodes and 8 images:
 // a lane has 8 nodes of one ring block (its share of G is one run of 64 bytes per
@@ -143,9 +143,9 @@ k_recon_radial(const float* __restrict__ R32m, const float2* __restrict__ Z, con
 // multiplied.  A chunk's sums are taken apart and then added, so that no sum is a
 // longer chain than in k_recon_radial (8 + K_m / 8 additions).  Bound by shared-memory
 // bandwidth and FP32 issue.  zm_reconstruct, us a call, with the sums split over
-// warps for eight images / like this: n_max 60 on 256 nodes, 64 images 24.3 / 15.6; 127
-// on 512, 16 images 30.0 / 23.6, 128 images 204 / 126; 300 on 512, 8 images 38.5 / 32.6,
-// 128 images 568 / 340; 1000 on 256, 16 images 381 / 175 (a thread per node before
+// warps for eight images / like this: n_max 60 on 256 nodes, 64 images 24.3 / 15.4; 127
+// on 512, 16 images 30.0 / 22.4, 128 images 204 / 125; 300 on 512, 8 images 38.5 / 30.4,
+// 128 images 568 / 327; 1000 on 256, 16 images 381 / 159 (a thread per node before
 // either: 16.9, 23.9, 131, 42.8, 390, 359).
 constexpr int RW_KC = 8, RW_STAGES = 3;
 
@@ -157,7 +157,7 @@ k_recon_radial_wide(const float* __restrict__ R32m, const float2* __restrict__ Z
     __shared__ __align__(16) float rows[RW_STAGES][RW_KC][NODES];
     __shared__ __align__(16) float2 zs[2][RW_KC][IMGS];
     const int i0 = blockIdx.x * NODES, m = blockIdx.y, b0 = blockIdx.z * IMGS;
-    const int Km = (n_max - m) / 2 + 1, chunks = (Km + RW_KC - 1) / RW_KC;
+    const int Km = (n_max - m) / 2 + 1;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int ig = warp % IG, nh = warp / IG;         // the warp's images and nodes
     const int ng = lane & 7, cg = lane >> 3;          // the lane's ring block and pair of images
@@ -166,16 +166,13 @@ k_recon_radial_wide(const float* __restrict__ R32m, const float2* __restrict__ Z
     // 16-byte words of a row: within 64 nodes the even ones first, then the odd
     // ones, so that the eight lanes of a phase read 128 consecutive bytes
     auto place = [](int q) { return (q & ~15) + ((q & 1) << 3) + ((q & 15) >> 1); };
-    // the first order of the c-th chunk taken: the high orders first, whose moments
-    // are the smaller ones wherever they fall off
-    auto order0 = [&](int c) { return (chunks - 1 - c) * RW_KC; };
-    auto issue = [&](int c) {
-        if (c < chunks) {
-            const int j0 = order0(c), live = min(RW_KC, Km - j0), st = c % RW_STAGES;
+    // chunks are taken from the high orders down, whose moments are the smaller ones
+    // wherever they fall off; orders past K_m in the first are zero rows and moments
+    auto issue = [&](int j0, int st) {
+        if (j0 >= 0) {
             for (int e = threadIdx.x; e < RW_KC * NODES / V; e += THREADS) {
                 const int k = e / (NODES / V), x = (e % (NODES / V)) * V;
-                if (k >= live) break;
-                const int on = i0 + x < n_rho;                        // else zero-filled
+                const int on = j0 + k < Km && i0 + x < n_rho;         // else zero-filled
                 const float* src = on ? Rm + (size_t)(j0 + k) * n_rho + x : Rm;
                 const uint32_t dst = rows_a + 4u * ((st * RW_KC + k) * NODES + 4 * place(x >> 2) + (x & 3));
                 if (V == 4)
@@ -190,54 +187,55 @@ k_recon_radial_wide(const float* __restrict__ R32m, const float2* __restrict__ Z
     };
     // one moment per thread and chunk: order t / IMGS of the chunk, image t mod IMGS
     const int zk = threadIdx.x / IMGS, zb = threadIdx.x % IMGS;
+    const bool zlive = zk < RW_KC && b0 + zb < batch;
     const float2* Zb = Z + (size_t)min(b0 + zb, batch - 1) * P;
-    auto moment = [&](int c) {
-        const int j = order0(c) + zk;
-        return c < chunks && zk < RW_KC && j < Km && b0 + zb < batch ? __ldg(Zb + moment_index(m + 2 * j, m)) : make_float2(0.f, 0.f);
+    auto moment = [&](int j0) {
+        return zlive && j0 >= 0 && j0 + zk < Km ? __ldg(Zb + moment_index(m + 2 * (j0 + zk), m)) : make_float2(0.f, 0.f);
     };
-    issue(0);                          // the table is the plan's
-    issue(1);
+    int j0 = ((Km + RW_KC - 1) / RW_KC - 1) * RW_KC;
+    issue(j0, 0);                      // the table is the plan's
+    issue(j0 - RW_KC, 1);
     griddep_wait();                    // the moments are written, G is free
     griddep_launch();
-    float2 zn = moment(0);
+    float2 zn = moment(j0);
     if (zk < RW_KC) zs[0][zk][zb] = zn;
-    zn = moment(1);
+    zn = moment(j0 - RW_KC);
     const bool busy = b0 + ig * 8 < batch && i0 + nh * 64 < n_rho;
     f32x2 tot[8][2];
 #pragma unroll
     for (int r = 0; r < 8; ++r) tot[r][0] = tot[r][1] = 0;
-    for (int c = 0; c < chunks; ++c) {
+    int st = 0, zbuf = 0;
+    for (; j0 >= 0; j0 -= RW_KC) {
         asm volatile("cp.async.wait_group 1;" ::: "memory");
-        __syncthreads();               // chunk c is here; chunk c - 1 is read
-        issue(c + 2);
-        if (zk < RW_KC) zs[(c + 1) & 1][zk][zb] = zn;
-        zn = moment(c + 2);
-        if (!busy) continue;
-        const int live = min(RW_KC, Km - order0(c));
-        const float* rk = &rows[c % RW_STAGES][0][nh * 64 + 4 * ng];
-        const float2* zk_ = &zs[c & 1][0][ig * 8 + cg * 2];
-        f32x2 acc[8][2];
+        __syncthreads();               // this chunk is here; the last one is read
+        issue(j0 - 2 * RW_KC, st + 2 < RW_STAGES ? st + 2 : st + 2 - RW_STAGES);
+        if (zk < RW_KC) zs[zbuf ^ 1][zk][zb] = zn;
+        zn = moment(j0 - 2 * RW_KC);
+        if (busy) {
+            const float* rk = &rows[st][0][nh * 64 + 4 * ng];
+            const float2* zr = &zs[zbuf][0][ig * 8 + cg * 2];
+            f32x2 acc[8][2];
 #pragma unroll
-        for (int r = 0; r < 8; ++r) acc[r][0] = acc[r][1] = 0;
+            for (int k = 0; k < RW_KC; ++k) {
+                const float4 a = *reinterpret_cast<const float4*>(rk + k * NODES);
+                const float4 b = *reinterpret_cast<const float4*>(rk + k * NODES + 32);
+                const ulonglong2 z = *reinterpret_cast<const ulonglong2*>(zr + k * IMGS);
+                const float r8[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
 #pragma unroll
-        for (int k = 0; k < RW_KC; ++k) {
-            if (k >= live) break;
-            const float4 a = *reinterpret_cast<const float4*>(rk + k * NODES);
-            const float4 b = *reinterpret_cast<const float4*>(rk + k * NODES + 32);
-            const ulonglong2 z = *reinterpret_cast<const ulonglong2*>(zk_ + k * IMGS);
-            const float r8[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+                for (int r = 0; r < 8; ++r) {
+                    const f32x2 rr = pack2(r8[r], r8[r]);
+                    acc[r][0] = k ? fma2(rr, z.x, acc[r][0]) : mul2(rr, z.x);
+                    acc[r][1] = k ? fma2(rr, z.y, acc[r][1]) : mul2(rr, z.y);
+                }
+            }
 #pragma unroll
             for (int r = 0; r < 8; ++r) {
-                const f32x2 rr = pack2(r8[r], r8[r]);
-                acc[r][0] = fma2(rr, z.x, acc[r][0]);
-                acc[r][1] = fma2(rr, z.y, acc[r][1]);
+                tot[r][0] = add2(tot[r][0], acc[r][0]);
+                tot[r][1] = add2(tot[r][1], acc[r][1]);
             }
         }
-#pragma unroll
-        for (int r = 0; r < 8; ++r) {
-            tot[r][0] = add2(tot[r][0], acc[r][0]);
-            tot[r][1] = add2(tot[r][1], acc[r][1]);
-        }
+        st = st + 1 < RW_STAGES ? st + 1 : 0;
+        zbuf ^= 1;
     }
     asm volatile("cp.async.wait_group 0;" ::: "memory");
     const int i = i0 + nh * 64 + ng * 8;
@@ -528,13 +526,21 @@ static int launch_radial(zm_plan_t p, const float* moments, int batch, unsigned 
         return launch_radial_tc(p, moments, batch, flags, G, st);
     }
     const bool vec = (p->n_rho & 3) == 0;
-    // more than four images: all orders in a warp, 256 nodes to a CTA, or 128 where
-    // rows are copied float by float (its copies are four times as many)
-    const int st_ = batch == 1   ? (vec ? launch_radial_t<1, 4> : launch_radial_t<1, 1>)(p, moments, batch, flags, G, st)
+    // More than four images: all orders in a warp once CTAs that split them would
+    // go several times around the device, the sooner the shorter the chain of orders
+    // is; 256 nodes to a CTA, or 128 where the grid has no more or rows are copied float
+    // by float.  zm_reconstruct, us a call, split / whole: n_max 200 on 128 nodes, 8
+    // images 14.6 / 18.9, on 512 nodes 24.5 / 22.5, 12 images 33.7 / 25.8; 300 on 64
+    // nodes, 11 images 17.6 / 23.2, on 512, 8 images 36.8 / 30.4; 100 on 256, 24 images
+    // 19.2 / 15.0; 30 on 256, 8 images 6.2 / 5.4.
+    const long long split = (long long)((p->n_rho + RR_NODES - 1) / RR_NODES) * (p->n_max + 1) * ((batch + 3) / 4);
+    const bool whole = batch > 4 && (p->n_max <= 30 || split > std::min(8 * p->n_max, 2400));
+    const int st_ = batch == 1 ? (vec ? launch_radial_t<1, 4> : launch_radial_t<1, 1>)(p, moments, batch, flags, G, st)
                     : batch == 2 ? (vec ? launch_radial_t<2, 4> : launch_radial_t<2, 1>)(p, moments, batch, flags, G, st)
-                    : batch <= 4 ? (vec ? launch_radial_t<4, 4> : launch_radial_t<4, 1>)(p, moments, batch, flags, G, st)
-                    : vec        ? launch_radial_wide_t<2, 4, 4>(p, moments, batch, flags, G, st)
-                                 : launch_radial_wide_t<2, 2, 1>(p, moments, batch, flags, G, st);
+                    : !whole     ? (vec ? launch_radial_t<4, 4> : launch_radial_t<4, 1>)(p, moments, batch, flags, G, st)
+                    : vec && p->n_rho > 256 ? launch_radial_wide_t<2, 4, 4>(p, moments, batch, flags, G, st)
+                    : vec ? launch_radial_wide_t<2, 2, 4>(p, moments, batch, flags, G, st)
+                          : launch_radial_wide_t<2, 2, 1>(p, moments, batch, flags, G, st);
     if (st_ != ZM_OK) return st_;
     *G_out = G;
     return ZM_OK;

@@ -1,4 +1,4 @@
-"""The FP32 radial reconstruction of more than four images, at the edges of its
+"""The FP32 radial reconstruction of larger batches, at the edges of its
 node tiles (256 nodes, 128 where rows are not 16-byte aligned), ring blocks, image
 groups of 16 and chunks of eight orders, through zm_reconstruct, against the oracle;
 an image alone, which takes the other kernel, agrees.
