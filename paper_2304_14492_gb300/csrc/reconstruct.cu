@@ -526,15 +526,15 @@ static int launch_radial(zm_plan_t p, const float* moments, int batch, unsigned 
         return launch_radial_tc(p, moments, batch, flags, G, st);
     }
     const bool vec = (p->n_rho & 3) == 0;
-    // More than four images: all orders in a warp once CTAs that split them would
-    // go several times around the device, the sooner the shorter the chain of orders
-    // is; 256 nodes to a CTA, or 128 where the grid has no more or rows are copied float
+    // More than four images: all orders in a warp, but past order 128 only once CTAs
+    // that split them would go several times around the device; 256 nodes to a CTA, or 128 where the grid has no more or rows are copied float
     // by float.  zm_reconstruct, us a call, split / whole: n_max 200 on 128 nodes, 8
     // images 14.6 / 18.9, on 512 nodes 24.5 / 22.5, 12 images 33.7 / 25.8; 300 on 64
     // nodes, 11 images 17.6 / 23.2, on 512, 8 images 36.8 / 30.4; 100 on 256, 24 images
-    // 19.2 / 15.0; 30 on 256, 8 images 6.2 / 5.4.
+    // 19.2 / 15.0; 30 on 256, 8 images 6.2 / 5.4; 108 on 77 nodes, 8 images 8.0 / 9.5, but
+    // 12.3 / 9.9 between the inverse transforms of 1024 angles.
     const long long split = (long long)((p->n_rho + RR_NODES - 1) / RR_NODES) * (p->n_max + 1) * ((batch + 3) / 4);
-    const bool whole = batch > 4 && (p->n_max <= 30 || split > std::min(8 * p->n_max, 2400));
+    const bool whole = batch > 4 && (p->n_max <= 128 || split > std::min(8 * p->n_max, 2400));
     const int st_ = batch == 1 ? (vec ? launch_radial_t<1, 4> : launch_radial_t<1, 1>)(p, moments, batch, flags, G, st)
                     : batch == 2 ? (vec ? launch_radial_t<2, 4> : launch_radial_t<2, 1>)(p, moments, batch, flags, G, st)
                     : !whole     ? (vec ? launch_radial_t<4, 4> : launch_radial_t<4, 1>)(p, moments, batch, flags, G, st)
