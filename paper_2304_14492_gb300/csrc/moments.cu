@@ -30,6 +30,7 @@ struct KbParams {
     float* fhat_out;       // [batch_total][n_rho][N] or NULL
     const float* fhat_in;  // [batch_total][n_rho][N] (polar input mode)
     int discard_in;        // fhat_in is the plan's scratch: its L2 lines are dropped once read
+    int release;           // the next kernel may start early (k_ring_spectra)
     GeoImage img[KB_MAX_IMG];
 };
 
@@ -150,7 +151,7 @@ __global__ void __launch_bounds__(256, kb_ctas(LOGN, MODE)) k_ring_spectra(const
         }
     };
     griddep_wait();                // the images or polar samples are written, the spectra are free
-    griddep_launch();              // (the grid is resident at once)
+    if (p.release) griddep_launch();
     if (POLAR && (int)blockIdx.x < n_items) load_ring(blockIdx.x);
     bool ready = false;
     for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
@@ -545,10 +546,11 @@ static int pick_rings(zm_plan_t p, int batch, bool tiled) {
     const int want = 2 * num_sms(p->device);
     // two rings to a CTA spread small calls over the SMs; rings of 512 angles and
     // more keep four (their twiddle tables are loaded by every CTA: one 2160 x
-    // 2160 image on 1024 x 1024, FP32, 20.8 us against 23.7 with two), but after the
-    // tiles only where the rings are few (one 2160 x 2160 image on 256 x 2048 10.8
-    // us against 11.7; one 1024 x 1024 image on 512 x 2048 18.2 against 14.0 with two)
-    const int least = p->n_theta >= 512 && !(tiled && (long long)p->n_rho * batch > want) ? 4 : 2;
+    // 2160 image on 1024 x 1024, gathered, FP32, 20.8 us against 23.7 with two), but of
+    // 1024 angles after the tiles only where the rings are few (the same call by the
+    // tiles 21.6 us with four, 19.7 with two)
+    const bool many = tiled && p->n_theta == 1024 && (long long)p->n_rho * batch > want;
+    const int least = p->n_theta >= 512 && !many ? 4 : 2;
     while (R > least && ((p->n_rho + R - 1) / R) * batch < want) R >>= 1;
     return R;
 }
@@ -578,6 +580,7 @@ static int launch_gather(zm_plan_t p, const zm_image_t* imgs, int b0, int nb, in
     kp.fhat_out = fhat_out;
     kp.fhat_in = nullptr;
     kp.discard_in = 0;
+    kp.release = 1;
     for (int c0 = b0; c0 < b0 + nb; c0 += KB_MAX_IMG) {
         const int nc = std::min(KB_MAX_IMG, b0 + nb - c0);
         kp.b_off = c0;
@@ -611,6 +614,10 @@ static int launch_polar_fft(zm_plan_t p, const float* fhat, int b0, int nb, int 
     kp.fhat_out = nullptr;
     kp.fhat_in = fhat;
     kp.discard_in = scratch && Fblk && ((uintptr_t)fhat & 127u) == 0 ? 1 : 0;
+    // spectra for the caller: what follows is the next call's tile resampler, which
+    // would take the SMs from rings still to come (four 596 x 1152 images on 282 x 512,
+    // captured: 15.0 us a call with, 10.5 without)
+    kp.release = Fblk || F == (const float*)p->ws_F.ptr || !tiled ? 1 : 0;
     for (int c0 = b0; c0 < b0 + nb; c0 += 65535) {
         const int nc = std::min(65535, b0 + nb - c0);
         kp.b_off = c0;
