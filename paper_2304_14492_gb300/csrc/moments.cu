@@ -478,7 +478,7 @@ static int launch_blk(int logn, const KbParams& kp, int nb, cudaStream_t st) {
 }
 
 template <int LOGN, int MODE>
-static int launch_kb_t(const KbParams& kp, int R, int nb, cudaStream_t st) {
+static int launch_kb_t(const KbParams& kp, int R, int nb, cudaStream_t st, bool early = true) {
     using FFT = RingFFT<LOGN>;
     const size_t smem = sizeof(float) * ((size_t)R * FFT::ROW_FLOATS +
                                          (MODE == KB_RESAMPLE ? 0 : (size_t)2 * (kp.n_max + 1) * R + 2)) +
@@ -507,14 +507,7 @@ static int launch_kb_t(const KbParams& kp, int R, int nb, cudaStream_t st) {
     k.nb = nb;
     const long long items = (long long)(kp.Fblk ? kp.n_chunks * (64 / R) : (kp.n_rho + R - 1) / R) * nb;
     const int grid = (int)std::min<long long>(items, (long long)per_sm * num_sms(dev));
-    // A gather of more than GATHER_PDL_SAMPLES is not launched early: it lives on
-    // L1, and CTAs that come in while the previous call's projection holds the SM's
-    // shared memory keep that split for their lifetime (zm_moments captured, with the
-    // early launch / without, us: 40 images of 1024 x 1024 on 512 x 256, bf16x3 149 / 54,
-    // fp16x3 151 / 69; 40 of 512 x 512 on 256 x 256, bf16x3 45 / 29; 1024 x 1024 on 512 x
-    // 1024, two images 26 / 17; half a million samples 0 to 13 % the same way, though
-    // uncaptured calls of that size gain 10 %).
-    if (MODE == KB_GATHER && (long long)nb * kp.n_rho * FFT::N > GATHER_PDL_SAMPLES) {
+    if (!early) {
         k_ring_spectra<LOGN, MODE><<<grid, R * 32, smem, st>>>(kp);
         ZM_LAUNCH_CHECK("k_ring_spectra");
         return ZM_OK;
@@ -524,17 +517,17 @@ static int launch_kb_t(const KbParams& kp, int R, int nb, cudaStream_t st) {
 }
 
 template <int MODE>
-static int launch_kb_mode(int logn, const KbParams& kp, int R, int nb, cudaStream_t st) {
+static int launch_kb_mode(int logn, const KbParams& kp, int R, int nb, cudaStream_t st, bool early = true) {
     switch (logn) {
-        case 3: return launch_kb_t<3, MODE>(kp, R, nb, st);
-        case 4: return launch_kb_t<4, MODE>(kp, R, nb, st);
-        case 5: return launch_kb_t<5, MODE>(kp, R, nb, st);
-        case 6: return launch_kb_t<6, MODE>(kp, R, nb, st);
-        case 7: return launch_kb_t<7, MODE>(kp, R, nb, st);
-        case 8: return launch_kb_t<8, MODE>(kp, R, nb, st);
-        case 9: return launch_kb_t<9, MODE>(kp, R, nb, st);
-        case 10: return launch_kb_t<10, MODE>(kp, R, nb, st);
-        case 11: return launch_kb_t<11, MODE>(kp, R, nb, st);
+        case 3: return launch_kb_t<3, MODE>(kp, R, nb, st, early);
+        case 4: return launch_kb_t<4, MODE>(kp, R, nb, st, early);
+        case 5: return launch_kb_t<5, MODE>(kp, R, nb, st, early);
+        case 6: return launch_kb_t<6, MODE>(kp, R, nb, st, early);
+        case 7: return launch_kb_t<7, MODE>(kp, R, nb, st, early);
+        case 8: return launch_kb_t<8, MODE>(kp, R, nb, st, early);
+        case 9: return launch_kb_t<9, MODE>(kp, R, nb, st, early);
+        case 10: return launch_kb_t<10, MODE>(kp, R, nb, st, early);
+        case 11: return launch_kb_t<11, MODE>(kp, R, nb, st, early);
         default: return set_error(ZM_EUNSUPPORTED, "n_theta 2^%d", logn);
     }
 }
@@ -585,8 +578,22 @@ static int launch_gather(zm_plan_t p, const zm_image_t* imgs, int b0, int nb, in
         const int nc = std::min(KB_MAX_IMG, b0 + nb - c0);
         kp.b_off = c0;
         for (int j = 0; j < nc; ++j) kp.img[j] = resolve(imgs[c0 + j]);
-        const int s = resample_only ? launch_kb_mode<KB_RESAMPLE>(p->log_theta, kp, R, nc, st)
-                                    : launch_kb_mode<KB_GATHER>(p->log_theta, kp, R, nc, st);
+        // A large gather is not launched early: it lives on L1, and CTAs that come in
+        // while the previous call's projection holds the SM's shared memory keep that
+        // split for their lifetime (zm_moments captured, with the early launch / without,
+        // us: 40 images of 1024 x 1024 on 512 x 256, bf16x3 149 / 54, fp16x3 151 / 69; 40 of
+        // 512 x 512 on 256 x 256, bf16x3 45 / 29; 1024 x 1024 on 512 x 1024, two images 26 /
+        // 17; half a million samples up to 30 % the same way, though calls of that size that
+        // are not captured gain as much).  The FP32 projection of few orders holds less of
+        // it: twice the samples up to order 64 and 256 angles (half a million: captured
+        // 0.88 to 1.05 of the time, else 0.74 to 0.93; order 100: 1.23 and 1.04).
+        const long long limit =
+            p->prec == PREC_FP32 && p->n_theta <= 256 && p->n_max <= 64 ? 2 * GATHER_PDL_SAMPLES : GATHER_PDL_SAMPLES;
+        const long long samples = (long long)nc * p->n_rho * p->n_theta;
+        const bool early = samples <= limit;
+        const int s = resample_only
+                          ? launch_kb_mode<KB_RESAMPLE>(p->log_theta, kp, R, nc, st, samples <= 8 * GATHER_PDL_SAMPLES)
+                          : launch_kb_mode<KB_GATHER>(p->log_theta, kp, R, nc, st, early);
         if (s != ZM_OK) return s;
     }
     return ZM_OK;
@@ -638,13 +645,18 @@ static int launch_polar_fft(zm_plan_t p, const float* fhat, int b0, int nb, int 
 // image side on N_rho x N_theta):
 //  256 angles: 256 on 128 x 256, 16 images 11.6 / 13.8; 700 on 350 x 256, 6 images
 //   12.8 / 17.4, 16 images 20.7 / 21.9; 1024 on 512 x 256, 6 images 15.7 / 19.5, 12
-//   images 22.5 / 25.1; 2160 on 1080 x 256, 4 images 21.9 / 27.6.  Only on grids of
-//   2^16 samples and about a million samples a call is the staged kernel ahead: 512
-//   on 256 x 256, 12 images 14.8 / 16.1, 16 images 17.1 / 16.2 (order 100: 19.5 /
-//   17.7), 40 images 29.1 / 33.1.
-//  512 angles (16 samples a lane), grids of up to 2^17 samples, up to 1.5 million a
-//   call: 512 on 256 x 512, 4 images 12.9 / 16.5, 8 images 17.3 / 16.9, 16 images
-//   25.5 / 21.7; FP32 16.3 / 19.3 and 23.6 / 21.4 with 8 and 16.
+//   images 22.5 / 25.1; 2160 on 1080 x 256, 4 images 21.9 / 27.6.  Only on grids of up
+//   to 2^16 samples and from about a million samples a call is the staged kernel ahead:
+//   512 on 256 x 256, order 50, 12 images 14.8 / 16.1, 16 images 17.1 / 16.2, 24 images
+//   21.6 / 22.5; 512 x 440 on 239 x 256, order 87 (more operand blocks to write), 20
+//   images 22.1 / 17.8, 40 images 32.7 / 29.8.  Its rows do not fit the stages where
+//   the image is large for the grid, which leaves the tiles: 1024 on 250 x 256, 16
+//   images 21.8 / 23.9, 40 images 48.5 / 42.1.
+//  512 angles (16 samples a lane), grids of up to 2^17 samples: FP32 rows up to 1.5
+//   million a call (512 on 256 x 512, 8 images 16.3 / 19.3, 16 images 23.6 / 21.4), operand
+//   blocks up to half a million (256 on 128 x 512, 8 images 13.6 / 14.8, 16 images 17.9
+//   / 15.8; 528 x 168 on 98 x 512, order 232, 20 images 22.2 / 16.9), or as far where the
+//   image is large for the grid (512 on 64 x 512, 24 images 18.5 / 23.0).
 //  1024 angles.  Grids of up to 2^17 samples would be staged, which is far slower
 //   there: up to 1.5 million a call (512 on 128 x 1024, 12 images 22.6 / 25.3, FP32
 //   20.5 / 25.7).  Larger grids have the tiles, and the form the spectra are wanted in
@@ -656,12 +668,18 @@ static int launch_polar_fft(zm_plan_t p, const float* fhat, int b0, int nb, int 
 //   1 image 21.3 / 18.9).
 // A plan told to fuse or not to (ZM_FUSED), or to use a tensor-core transform, does
 // that.
-static bool gather_by_default(zm_plan_t p, int batch, bool operand_blocks) {
+static bool gather_by_default(zm_plan_t p, const zm_image_t& im, int batch, bool operand_blocks) {
     if (p->fused_mode != 0 || p->dft_mode > 0 || p->pdft_mode > 0) return false;
     const long long samples = (long long)p->n_rho * p->n_theta, call = samples * batch;
+    const long long area = (long long)im.height * im.width;
     if (p->n_theta < 256) return true;
-    if (p->n_theta == 256) return samples > 1 << 16 || call <= 7ll << 17 || call > 3ll << 19;
-    if (p->n_theta == 512) return samples <= FUSED_AUTO_SAMPLES && call <= 3ll << 19;
+    if (p->n_theta == 256) {
+        if (samples > 1 << 16) return true;
+        if (area > 12 * samples) return call <= 1ll << 21;
+        return call <= 7ll << 17 || call > (operand_blocks && p->n_max > 64 ? 5ll << 19 : 3ll << 19);
+    }
+    if (p->n_theta == 512)
+        return samples <= FUSED_AUTO_SAMPLES && call <= (operand_blocks && area <= 4 * samples ? 1ll << 19 : 3ll << 19);
     if (p->n_theta > 1024) return false;
     if (samples <= FUSED_AUTO_SAMPLES) return call <= 3ll << 19;
     return operand_blocks ? call <= 5ll << 18 : call < 1ll << 20;
@@ -681,7 +699,8 @@ int launch_spectra(zm_plan_t p, const zm_image_t* imgs, const float* fhat_in, in
     if (fhat_in) return launch_polar_fft(p, fhat_in, 0, batch, batch, F, Fblk, st);
     const bool fuse = p->fused_mode > 0 ||
                       (p->fused_mode == 0 && (long long)p->n_rho * p->n_theta <= FUSED_AUTO_SAMPLES);
-    const bool gather = p->tune_gather == 1 || (p->tune_gather == 0 && !resample_only && gather_by_default(p, batch, Fblk != nullptr));
+    const bool gather = p->tune_gather == 1 || (p->tune_gather == 0 && !resample_only &&
+                                                gather_by_default(p, imgs[0], batch, Fblk != nullptr));
     const bool dft = Fblk && !fhat_out && !resample_only && !gather && p->dft_mode > 0;
     auto use_dft = [&](int b) { return dft && dft_eligible(p, imgs[b]); };
     auto use_fused = [&](int b) { return fuse && !resample_only && !gather && fused_eligible(p, imgs[b]); };

@@ -352,6 +352,7 @@ constexpr int RED_MAX_PARTS = 1024;   // parts (records) per image of the pixel 
 constexpr int KD_MAX_IMG = 128;       // images per launch of the pixel passes
 
 constexpr long long GATHER_PDL_SAMPLES = 1ll << 18;   // largest gather (samples) launched before its predecessor ends
+                                                      // (launch_gather; twice as many with an FP32 projection of few orders)
 
 // Cartesian-tile resampling (resample_tiles.cu)
 bool tma_eligible(const zm_image_t& im);

@@ -1,5 +1,5 @@
 """Calls on both sides of the lines at which the default route changes (gather,
-staged, tiles, by angles, samples an image and samples a call): the same spectra and
+staged, tiles, by angles, samples an image and a call, image size, order and form): the same spectra and
 moments as on plans told to stage or to tile, and the route told by its launches
 (gathered and staged spectra are one kernel, tiles and ring FFT two; the staged
 kernel alone builds a list, seen as nothing launched for it, and is told from the
@@ -47,22 +47,25 @@ def run(imgs, n_max, n_rho, n_theta, prec):
     return out, F, n
 
 
-# (side, n_rho, n_theta, batch, tiles for moments with blocks, tiles for FP32 rows)
-CASES = [(128, 64, 128, 3, False, False),
-         (128, 256, 256, 14, False, False), (128, 256, 256, 15, False, False),    # 7/8 million: gathered, staged
-         (128, 256, 256, 24, False, False), (128, 256, 256, 25, False, False),    # 1.5 million: staged, gathered
-         (128, 320, 256, 12, False, False),                                       # a grid above 2^16: gathered
-         (128, 256, 512, 12, False, False), (128, 256, 512, 13, False, False),    # 1.5 million: gathered, staged
-         (128, 257, 512, 1, True, True),                                          # a grid above 2^17: tiles
-         (128, 128, 1024, 12, False, False), (128, 128, 1024, 13, False, False),  # 1.5 million: gathered, staged
-         (128, 129, 1024, 7, False, False), (128, 256, 1024, 4, False, True),     # a million: FP32 rows by tiles
-         (128, 256, 1024, 5, False, True), (128, 256, 1024, 6, True, True),       # 1.25 million: tiles
-         (128, 16, 2048, 1, False, False), (128, 65, 2048, 1, True, True)]        # 2048: staged, tiles
+# (side, n_max, n_rho, n_theta, batch, tiles for moments with blocks, tiles for FP32 rows)
+CASES = [(128, 30, 64, 128, 3, False, False),
+         (128, 30, 256, 256, 14, False, False), (128, 30, 256, 256, 15, False, False),  # 7/8 million: gathered, staged
+         (128, 30, 256, 256, 24, False, False), (128, 30, 256, 256, 25, False, False),  # 1.5 million: staged, gathered
+         (128, 65, 256, 256, 25, False, False), (128, 65, 256, 256, 41, False, False),  # order 65, 2.5 million: blocks staged, gathered
+         (128, 30, 320, 256, 12, False, False),                                         # a grid above 2^16: gathered
+         (1024, 30, 256, 256, 32, False, False), (1024, 30, 256, 256, 33, True, True),  # large images, 2 million: gathered, tiles
+         (128, 30, 256, 512, 4, False, False), (128, 30, 256, 512, 5, False, False),    # blocks, half a million: gathered, staged
+         (128, 30, 256, 512, 12, False, False), (128, 30, 256, 512, 13, False, False),  # FP32 rows, 1.5 million: gathered, staged
+         (400, 30, 64, 512, 17, False, False),                                          # large images, blocks: gathered
+         (128, 30, 257, 512, 1, True, True),                                            # a grid above 2^17: tiles
+         (128, 30, 128, 1024, 12, False, False), (128, 30, 128, 1024, 13, False, False),  # 1.5 million: gathered, staged
+         (128, 30, 129, 1024, 7, False, False), (128, 30, 256, 1024, 4, False, True),   # a million: FP32 rows by tiles
+         (128, 30, 256, 1024, 5, False, True), (128, 30, 256, 1024, 6, True, True),     # 1.25 million: tiles
+         (128, 30, 16, 2048, 1, False, False), (128, 30, 65, 2048, 1, True, True)]      # 2048: staged, tiles
 
 
-@pytest.mark.parametrize("side,n_rho,n_theta,batch,tiles_blk,tiles_f32", CASES)
-def test_both_sides_of_every_line(side, n_rho, n_theta, batch, tiles_blk, tiles_f32, monkeypatch):
-    n_max = 30
+@pytest.mark.parametrize("side,n_max,n_rho,n_theta,batch,tiles_blk,tiles_f32", CASES)
+def test_both_sides_of_every_line(side, n_max, n_rho, n_theta, batch, tiles_blk, tiles_f32, monkeypatch):
     gen = torch.Generator(device=DEV)
     gen.manual_seed(n_rho * n_theta + batch)
     imgs = [torch.rand((side, side), device=DEV, generator=gen) for _ in range(batch)]
