@@ -649,14 +649,15 @@ static int launch_polar_fft(zm_plan_t p, const float* fhat, int b0, int nb, int 
 //   to 2^16 samples and from about a million samples a call is the staged kernel ahead:
 //   512 on 256 x 256, order 50, 12 images 14.8 / 16.1, 16 images 17.1 / 16.2, 24 images
 //   21.6 / 22.5; 512 x 440 on 239 x 256, order 87 (more operand blocks to write), 20
-//   images 22.1 / 17.8, 40 images 32.7 / 29.8.  Its rows do not fit the stages where
-//   the image is large for the grid, which leaves the tiles: 1024 on 250 x 256, 16
+//   images 22.1 / 17.8, 40 images 32.7 / 29.8; with the fp16 projection already from
+//   half a million, 872 x 268 on 145 x 256, 18 images 22.5 / 21.4.  Its rows do not fit the stages where
+//   the disk is large for the grid, which leaves the tiles: 1024 on 250 x 256, 16
 //   images 21.8 / 23.9, 40 images 48.5 / 42.1.
 //  512 angles (16 samples a lane), grids of up to 2^17 samples: FP32 rows up to 1.5
 //   million a call (512 on 256 x 512, 8 images 16.3 / 19.3, 16 images 23.6 / 21.4), operand
 //   blocks up to half a million (256 on 128 x 512, 8 images 13.6 / 14.8, 16 images 17.9
 //   / 15.8; 528 x 168 on 98 x 512, order 232, 20 images 22.2 / 16.9), or as far where the
-//   image is large for the grid (512 on 64 x 512, 24 images 18.5 / 23.0).
+//   disk is large for the grid (512 on 64 x 512, 24 images 18.5 / 23.0).
 //  1024 angles.  Grids of up to 2^17 samples would be staged, which is far slower
 //   there: up to 1.5 million a call (512 on 128 x 1024, 12 images 22.6 / 25.3, FP32
 //   20.5 / 25.7).  Larger grids have the tiles, and the form the spectra are wanted in
@@ -671,12 +672,14 @@ static int launch_polar_fft(zm_plan_t p, const float* fhat, int b0, int nb, int 
 static bool gather_by_default(zm_plan_t p, const zm_image_t& im, int batch, bool operand_blocks) {
     if (p->fused_mode != 0 || p->dft_mode > 0 || p->pdft_mode > 0) return false;
     const long long samples = (long long)p->n_rho * p->n_theta, call = samples * batch;
-    const long long area = (long long)im.height * im.width;
+    const GeoImage g = resolve(im);
+    const double area = 4.0 * g.r * g.r;                 // of the disk's square, in pixels
     if (p->n_theta < 256) return true;
     if (p->n_theta == 256) {
         if (samples > 1 << 16) return true;
         if (area > 12 * samples) return call <= 1ll << 21;
-        return call <= 7ll << 17 || call > (operand_blocks && p->n_max > 64 ? 5ll << 19 : 3ll << 19);
+        return call <= (p->prec == PREC_FP16X3 ? 1ll << 19 : 7ll << 17) ||
+               call > (operand_blocks && p->n_max > 64 ? 5ll << 19 : 3ll << 19);
     }
     if (p->n_theta == 512)
         return samples <= FUSED_AUTO_SAMPLES && call <= (operand_blocks && area <= 4 * samples ? 1ll << 19 : 3ll << 19);

@@ -273,30 +273,43 @@ __global__ void __launch_bounds__(TC_THREADS) k_project_tc(const __grid_constant
     }
 }
 
-// Sums of the S slices and the Neumann factor: a thread per (row, image), images
-// fastest, so that a warp reads whole lines of every slice; the one scattered access
-// is the write.  (With a thread per output, consecutive moments, each read its own
+// Sums of the S slices and the Neumann factor.  ROWS: a thread per (row, image),
+// images fastest, so that a warp reads whole lines of every slice; the one scattered
+// access is the write.  (With a thread per output, consecutive moments, each read its own
 // sector of every slice, which needed the L1 that an early launch, beside the
 // projection's shared memory, does not have: bf16, n_max 127 on 512 nodes, 64 images
 // 52.5 us a call with the early launch and 41.9 without, now 28.8; 60 on 501 nodes, 32
-// images 19.3, 16.5 and 11.4; 12 on 64 nodes, 1 image 5.7, 6.6 and 5.6.)
+// images 19.3, 16.5 and 11.4.)  Else a thread per output, where there are one or two
+// slices to read and the scattered writes cost more (order 182 on 49 nodes, one slice,
+// 64 images 1.27 of the time by rows, on 98, two slices, 1.11; order 60 on 128 0.94).
+template <bool ROWS>
 __global__ void __launch_bounds__(256)
-k_project_reduce_tc(const float* __restrict__ part, int S, int P, int ncol, const int* __restrict__ mrow, int n_max,
-                    int batch, int neumann, float* __restrict__ out) {
+k_project_reduce_tc(const float* __restrict__ part, int S, int P, int ncol, const int2* __restrict__ pair_nm,
+                    const int* __restrict__ mrow, int n_max, int batch, int neumann, float* __restrict__ out) {
     const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    // the row's order (rows are m-major), from the plan's tables
-    const int row = idx / batch, b = idx - row * batch;
-    int m = 0;
-    for (int hi = n_max + 1; hi - m > 1;) {             // the last m with mrow[m] <= row
-        const int mid = (m + hi) >> 1;
-        if (__ldg(&mrow[mid]) <= row) m = mid;
-        else hi = mid;
+    int row, b, m, q;
+    if (ROWS) {
+        // the row's order (rows are m-major), from the plan's tables
+        row = idx / batch;
+        b = idx - row * batch;
+        m = 0;
+        for (int hi = n_max + 1; hi - m > 1;) {         // the last m with mrow[m] <= row
+            const int mid = (m + hi) >> 1;
+            if (__ldg(&mrow[mid]) <= row) m = mid;
+            else hi = mid;
+        }
+        q = moment_index(m + 2 * (row - __ldg(&mrow[m])), m);
+    } else {
+        b = idx / P;
+        q = idx - b * P;
+        const int2 nm = __ldg(&pair_nm[q]);
+        m = nm.y;
+        row = __ldg(&mrow[m]) + (nm.x - m) / 2;
     }
-    const int n = m + 2 * (row - __ldg(&mrow[m]));
     griddep_wait();                    // the partial sums are written, out is free
     griddep_launch();
     if (idx >= batch * P) return;
-    const float2* ps = reinterpret_cast<const float2*>(part) + idx;
+    const float2* ps = reinterpret_cast<const float2*>(part) + (ROWS ? (size_t)idx : (size_t)row * batch + b);
     const size_t slice = (size_t)P * (ncol / 2);
     float re = 0.f, im = 0.f;
 #pragma unroll 8
@@ -306,7 +319,7 @@ k_project_reduce_tc(const float* __restrict__ part, int S, int P, int ncol, cons
         im += v.y;
     }
     const float f = (neumann && m == 0) ? 0.5f : 1.f;
-    float* o = out + ((size_t)b * P + moment_index(n, m)) * 2;
+    float* o = out + ((size_t)b * P + q) * 2;
     o[0] = re * f;
     o[1] = im * f;
 }
@@ -356,9 +369,10 @@ int launch_projection_tc(zm_plan_t p, const float* F, int batch, float* out, uns
     dim3 grid(p->n_max + 1, ctiles, S);
     ZM_LAUNCH_PDL("k_project_tc", k_project_tc, grid, dim3(TC_THREADS), smem, st, tp);
     const int tot = batch * p->P;
-    ZM_LAUNCH_PDL("k_project_reduce_tc", k_project_reduce_tc, dim3((tot + 255) / 256), dim3(256), 0, st,
-                  (const float*)tp.part, S, p->P, ncol, (const int*)p->mrow, p->n_max, batch,
-                  (flags & ZM_NEUMANN) ? 1 : 0, out);
+    const bool rows = S > 2 || (S == 2 && p->n_max < 128);
+    auto reduce = rows ? k_project_reduce_tc<true> : k_project_reduce_tc<false>;
+    ZM_LAUNCH_PDL("k_project_reduce_tc", reduce, dim3((tot + 255) / 256), dim3(256), 0, st, (const float*)tp.part, S, p->P,
+                  ncol, (const int2*)p->pair_nm, (const int*)p->mrow, p->n_max, batch, (flags & ZM_NEUMANN) ? 1 : 0, out);
     return ZM_OK;
 }
 

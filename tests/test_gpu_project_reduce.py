@@ -28,7 +28,8 @@ def _lib():
 
 
 @pytest.mark.parametrize("prec,split", [(zm.ZM_PREC_BF16X3, 3 * 2.0 ** -16), (zm.ZM_PREC_FP16X3, 3 * 2.0 ** -22)])
-@pytest.mark.parametrize("n_max,n_rho,n_theta", [(0, 5, 8), (1, 64, 8), (2, 65, 8), (3, 640, 8), (31, 128, 64), (64, 130, 256)])
+@pytest.mark.parametrize("n_max,n_rho,n_theta", [(0, 5, 8), (1, 64, 8), (2, 65, 8), (3, 640, 8), (31, 128, 64), (64, 130, 256),
+                                                 (130, 70, 512)])
 @pytest.mark.parametrize("batch,flags", [(1, 0), (3, zm.ZM_NEUMANN), (65, zm.ZM_NEUMANN), (257, 0)])
 def test_every_moment_in_its_place(n_max, n_rho, n_theta, batch, flags, prec, split):
     rng = np.random.default_rng(n_max * 1000 + batch)
