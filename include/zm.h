@@ -149,8 +149,8 @@ int zm_plan_nodes(zm_plan_t plan, double* rho, double* wr, void* stream);
  *  imgs  host array of `batch` device image descriptors (any sizes)
  *  out   device float[batch][P][2]
  *  flags ZM_NEUMANN divides each moment by eps_m (2 for m = 0, else 1; Eq. 14)
- * Path: grids of at most 256 angles, and smaller calls on 512 and 1024, are resampled
- * and ring-transformed in one kernel that gathers the pixels of each sample.
+ * Path: most grids of at most 256 angles, and smaller calls on 512 and 1024, are
+ * resampled and ring-transformed in one kernel that gathers the pixels of each sample.
  * Otherwise, images with a 16-byte aligned base and a pitch and width that are
  * multiples of 4 floats are resampled and ring-transformed in one kernel that
  * stages their rows (the polar samples stay on chip either way) when a plan has

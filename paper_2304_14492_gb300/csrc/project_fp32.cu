@@ -19,6 +19,7 @@
 // and a split over i reduced by a second kernel; now 16 us (cold, serialised).
 #include <algorithm>
 
+#include "packed.cuh"
 #include "tc_common.cuh"
 #include "zm_internal.cuh"
 
@@ -61,7 +62,7 @@ __device__ __forceinline__ void pf_stage(uint32_t dst, const float* src, int row
 // acc[j][c] += sum over a staged chunk of A[rg + 4 j][.] F[cg + 8 c][.]
 template <int TM, int TC>
 __device__ __forceinline__ void pf_chunk(const float* a, const float* f, int rg, int cg,
-                                         unsigned long long (&acc)[8][TC]) {
+                                         f32x2 (&acc)[8][TC]) {
 #pragma unroll 2
     for (int k = 0; k < PF_K; k += 4) {
         ulonglong2 av[TM], fv[TC];
@@ -75,8 +76,8 @@ __device__ __forceinline__ void pf_chunk(const float* a, const float* f, int rg,
         for (int j = 0; j < TM; ++j)
 #pragma unroll
             for (int c = 0; c < TC; ++c) {
-                asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc[j][c]) : "l"(av[j].x), "l"(fv[c].x));
-                asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc[j][c]) : "l"(av[j].y), "l"(fv[c].y));
+                acc[j][c] = fma2(av[j].x, fv[c].x, acc[j][c]);
+                acc[j][c] = fma2(av[j].y, fv[c].y, acc[j][c]);
             }
     }
 }
@@ -105,11 +106,11 @@ __global__ void __launch_bounds__(256) k_project_fp32(const __grid_constant__ Pf
     const float* A = p.A + (size_t)(p.mrow[m] + j0) * p.n_rho;
     const float* F = p.F + ((size_t)m * p.ncol + col0) * p.n_rho;
     const int chunks = (p.n_rho + PF_K - 1) / PF_K;
-    unsigned long long acc[8][TC];
+    f32x2 acc[8][TC];
 #pragma unroll
     for (int j = 0; j < 8; ++j)
 #pragma unroll
-        for (int c = 0; c < TC; ++c) acc[j][c] = 0ull;
+        for (int c = 0; c < TC; ++c) acc[j][c] = 0;
     auto stage_a = [&](int ch, int s) {
         if (ch < chunks) pf_stage<V>(buf_a + 4u * s * BUF, A, srow, live, ch * PF_K, p.n_rho, lane);
     };
@@ -145,7 +146,7 @@ __global__ void __launch_bounds__(256) k_project_fp32(const __grid_constant__ Pf
     for (int j = 0; j < 8; ++j)
 #pragma unroll
         for (int c = 0; c < TC; ++c) {
-            const float2 v = *reinterpret_cast<float2*>(&acc[j][c]);
+            const float2 v = unpack2(acc[j][c]);
             if (j < nj) buf[(rg + 4 * j) * RP + cg + 8 * c] = v.x + v.y;
         }
     __syncthreads();
