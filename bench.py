@@ -362,7 +362,7 @@ def stage_rooflines(zm, torch, dev, st, plan, descs, B, P, hbm, peaks, reps=100)
         t = event_loop(torch, st, lambda: zm.zm_stage_spectra(pf, descs, st), reps)
         res["K-b_fused"] = {"launch_ms": t, "achieved": kb / (t / 1000.0) / 1e9, "frac": kb / (t / 1000.0) / 1e9 / hbm,
                             "note": "the fused resampling + ring FFT kernel forced on this grid (ZM_FUSED=1); "
-                                    "zm_moments tiles grids of more than 2^17 polar samples per image"}
+                                    "zm_moments tiles batches of this grid"}
     finally:
         zm.zm_plan_destroy(pf)
     for key, name in (("K-b", "kb_tile_4k_b16" if kb_launches > 1 else "kb_fused_4k_b16"),
