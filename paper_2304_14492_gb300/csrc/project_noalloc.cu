@@ -15,7 +15,8 @@
 using namespace zm;
 
 // The largest request, P(n_max) * 2 * batch floats, that the interface takes: the
-// size of the fixed scratch an earlier form of this call kept.
+// size of the fixed scratch an earlier form of this call kept.  Nothing here needs
+// the limit any more; it stays because requests that were refused stay refused.
 constexpr size_t NOALLOC_FLOATS = (size_t)1 << 21;
 
 extern "C" int zm_project_noalloc(zm_plan_t plan, const float* spectra, int batch, float* out, unsigned flags,
@@ -26,8 +27,8 @@ extern "C" int zm_project_noalloc(zm_plan_t plan, const float* spectra, int batc
     const size_t floats = (size_t)plan->P * 2 * batch;
     if (floats > NOALLOC_FLOATS)
         return set_error(ZM_EINVAL,
-                         "zm_project_noalloc: P(n_max) * 2 * batch = %zu floats exceeds the %zu floats (a fixed scratch size) "
-                         "this call is specified for; use a smaller batch or zm_project",
+                         "zm_project_noalloc: P(n_max) * 2 * batch = %zu floats exceeds the %zu floats this call takes (the "
+                         "limit of the fixed scratch it once kept); use a smaller batch or zm_project",
                          floats, NOALLOC_FLOATS);
     DeviceGuard g(plan->device);
     if (!g.ok) return set_error(ZM_ECUDA, "cannot select device %d", plan->device);
